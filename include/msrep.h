@@ -225,7 +225,8 @@ msrep_status msrep_spmv_workspace_size(const msrep_matrix *A,
                                        size_t *bytes);
 
 /* flags for msrep_spmv */
-#define MSREP_COMP_ALL 0x10u  /* low precision: compensate every row      */
+#define MSREP_COMP_ALL 0x10u  /* low precision: compensate every row (this
+                                  version does so by default)              */
 #define MSREP_COMP_NONE 0x20u /* low precision: plain FP32 accumulation   */
 #define MSREP_STREAM_TMA 0x40u /* stage the nonzeros through shared memory
                                   with bulk copies (TMA) instead of direct
@@ -251,9 +252,9 @@ msrep_status msrep_spmv_workspace_size(const msrep_matrix *A,
  *
  * Types: val_dtype F64 with xy_dtype F64 (the plain path), or val_dtype F32
  * or BF16 with xy_dtype F32 (the low-precision form: FP32 products, FP32
- * accumulation with TwoSum compensation on rows longer than 256 nonzeros
- * and on rows split between thread-block tiles, partial sums of split rows
- * merged in FP64).  x has n entries, y has m entries, device memory.
+ * accumulation with TwoSum compensation: of rows longer than 256 nonzeros and
+ * of rows split between thread-block tiles always, and in this version of
+ * every row; partial sums of split rows merged in FP64).  x has n entries, y has m entries, device memory.
  *
  * Merge: every row split by a partition (or tile) boundary gets
  * alpha * (sum of its partials, in partition order) + beta * y_in, beta

@@ -49,11 +49,11 @@ __device__ __forceinline__ int owner_item(const int64_t *toff, int count, int64_
 
 // W warps per block; dynamic shared memory: per warp the row pointers of
 // its tile, rp_cap = largest tile + 8 entries.
-template <class Pol, int W>
+template <class Pol, int W, bool kComp>
 __global__ void __launch_bounds__(BShape<W>::kThreads, BShape<W>::kMinBlocks)
     batched_csr(const BatchItem *items, const int64_t *toff, int count, const void *const *xs,
                 void *const *ys, double *head, double *tail, double alpha, double beta,
-                int finish, unsigned comp_mode, int *err, int rp_cap) {
+                int finish, int *err, int rp_cap) {
   extern __shared__ __align__(16) int32_t s_rp_all[];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t *s_rp = s_rp_all + wid * rp_cap;
@@ -86,15 +86,17 @@ __global__ void __launch_bounds__(BShape<W>::kThreads, BShape<W>::kMinBlocks)
     a.head = head + base;
     a.tail = tail + base;
     a.m = it.m;
-    a.comp_mode = comp_mode;
+    a.comp_mode = 0;
     a.err = err;
     const int32_t r0 = __ldg(a.tile_row + b), k0 = __ldg(a.tile_k + b);
     const int32_t r1 = __ldg(a.tile_row + b + 1), k1 = __ldg(a.tile_k + b + 1);
     const int32_t rend = min(r1 + 2, a.m + 1);
     for (int32_t r = r0 + lane; r < rend; r += 32) s_rp[r - r0] = __ldg(a.row_ptr + r);
     __syncwarp();
-    csr_tile_compute<Pol>(a, b, r0, k0, r1, k1, s_rp, Seg<int32_t>{a.col_idx, 0},
-                          Seg<typename Pol::V>{a.val, 0}, it.nnz, GlobalSrc{});
+    csr_tile_compute<Pol, GlobalSrc, false, kComp>(a, b, r0, k0, r1, k1, s_rp,
+                                                   Seg<int32_t>{a.col_idx, 0},
+                                                   Seg<typename Pol::V>{a.val, 0}, it.nnz,
+                                                   GlobalSrc{});
     __syncwarp();
   }
 }
@@ -117,6 +119,7 @@ __global__ void batched_fixup(const BatchItem *items, const int64_t *toff, int c
         r = __ldg(tile_row + b);
         f = __ldg(row_ptr + r) < __ldg(tile_k + b);
       }
+      __device__ bool continues(int b, int32_t r) const { return __ldg(tile_row + b) == r; }
     } v{it.tile_row, it.tile_k, it.row_ptr};
     fixup_tile(v, T, static_cast<int>(g - base), head + base, tail + base,
                static_cast<X *>(ys[j]), alpha, beta);
@@ -194,7 +197,7 @@ msrep_status launch_batched(const BatchItem *items, const int64_t *toff, int cou
   if (!tile_supported(max_tile))
     return fail(MSREP_ERR_INVALID_ARG, "unsupported largest tile %d", max_tile);
   const int finish = finish_mode(alpha, beta);
-  const unsigned comp = flags & (MSREP_COMP_ALL | MSREP_COMP_NONE);
+  const bool plain = (flags & (MSREP_COMP_ALL | MSREP_COMP_NONE)) == MSREP_COMP_NONE;
   const int64_t T = total_tiles;
   if (T == 0) return MSREP_OK;
   const int sms = sm_count();
@@ -237,18 +240,25 @@ msrep_status launch_batched(const BatchItem *items, const int64_t *toff, int cou
     const int64_t grid =
         std::max<int64_t>(1, std::min<int64_t>(ceil_div(T, warps), int64_t(nb) * sms));
     kern<<<static_cast<int>(grid), threads, smem, st>>>(items, toff, count, xs, ys, head, tail,
-                                                        alpha, beta, finish, comp, err, rp_cap);
+                                                        alpha, beta, finish, err, rp_cap);
     MSREP_CUDA_TRY(cudaGetLastError());
     const int64_t fg = std::max<int64_t>(1, std::min<int64_t>(ceil_div(T, 256), 4 * sms));
     MSREP_TRY(launch_dependent(fix, fg, 256, st, 0, items, toff, count, ys, head, tail, alpha,
                                beta));
     return MSREP_OK;
   };
+  auto shape = [&](auto pol, auto comp, auto fix) -> msrep_status {
+    using Pol = decltype(pol);
+    constexpr bool kComp = decltype(comp)::value;
+    if (cta_threads == 128) return launch(batched_csr<Pol, 4, kComp>, fix, 4, BShape<4>::kMinBlocks);
+    if (cta_threads == 512)
+      return launch(batched_csr<Pol, 16, kComp>, fix, 16, BShape<16>::kMinBlocks);
+    return launch(batched_csr<Pol, 8, kComp>, fix, 8, BShape<8>::kMinBlocks);
+  };
   auto shaped = [&](auto pol, auto fix) -> msrep_status {
     using Pol = decltype(pol);
-    if (cta_threads == 128) return launch(batched_csr<Pol, 4>, fix, 4, BShape<4>::kMinBlocks);
-    if (cta_threads == 512) return launch(batched_csr<Pol, 16>, fix, 16, BShape<16>::kMinBlocks);
-    return launch(batched_csr<Pol, 8>, fix, 8, BShape<8>::kMinBlocks);
+    if (!Pol::kLow || plain) return shape(pol, std::false_type{}, fix);
+    return shape(pol, std::integral_constant<bool, Pol::kLow>{}, fix);
   };
   switch (val_dtype) {
     case MSREP_F64: return shaped(PolF64{}, batched_fixup<double>);

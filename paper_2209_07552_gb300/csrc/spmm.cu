@@ -19,49 +19,57 @@ msrep_status check_matrix(const msrep_matrix *A);
 int32_t effective_tile(int32_t tile);
 
 // xt[c * KP + j] = x[j * ldx + c] for j < k, 0 for k <= j < KP; a thread
-// per column: coalesced reads of each vector, one KP-wide write
+// per column: coalesced reads of each vector, the row written as 16-byte
+// stores where it is that wide (xt is 32-byte aligned)
 template <class X, int KP>
 __device__ __forceinline__ void interleave_column(const X *x, int64_t ldx, int k, int64_t c,
                                                   X *xt) {
-  X r[KP];
+  alignas(16) X r[KP];
 #pragma unroll
   for (int j = 0; j < KP; ++j) r[j] = j < k ? x[j * ldx + c] : X(0);
+  if constexpr (KP * sizeof(X) >= 16) {
 #pragma unroll
-  for (int j = 0; j < KP; ++j) xt[c * KP + j] = r[j];
+    for (int j = 0; j < KP * int(sizeof(X)) / 16; ++j)
+      reinterpret_cast<int4 *>(xt + c * KP)[j] = reinterpret_cast<const int4 *>(r)[j];
+  } else {
+#pragma unroll
+    for (int j = 0; j < KP; ++j) xt[c * KP + j] = r[j];
+  }
 }
 
 template <class X, int KP>
 __global__ void interleave_x(const X *x, int64_t ldx, int k, int64_t n, X *xt) {
+  grid_dependency_wait();
   for (int64_t c = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; c < n;
        c += int64_t(gridDim.x) * blockDim.x)
     interleave_column<X, KP>(x, ldx, k, c, xt);
 }
 
 template <class Pol, int KP>
-__global__ void __launch_bounds__(kKvThreads) csr_spmm_direct(SpmmArgs<Pol, KP> a,
-                                                              const int32_t *n_tiles,
-                                                              int64_t nnz) {
-  using Sh = KvShape<typename Pol::X, KP>;
-  __shared__ KvSmem<typename Pol::Acc, Sh::G> sm;
+__global__ void __launch_bounds__(kKvThreads, KvShape<typename Pol::X, KP>::kBlocks)
+    csr_spmm_direct(SpmmArgs<Pol> a, const int32_t *n_tiles) {
+  using X = typename Pol::X;
+  __shared__ KvWarpSmem<X, KvShape<X, KP>::VW> sm[kKvWarps];
   grid_dependency_wait();
-  const int T = *n_tiles, ts = threadIdx.x / Sh::GT;
-  // alpha = 1, beta = 0 finishes rows by a copy, chosen at compile time
-  if (a.finish == kFinishCopy) {
-    for (int b = blockIdx.x * Sh::G + ts; b < T; b += gridDim.x * Sh::G)
-      kv_tile<Pol, KP, Sh::G, true>(a, b, nnz, sm, ts);
-  } else {
-    for (int b = blockIdx.x * Sh::G + ts; b < T; b += gridDim.x * Sh::G)
-      kv_tile<Pol, KP, Sh::G>(a, b, nnz, sm, ts);
-  }
+  const int T = *n_tiles, wid = threadIdx.x >> 5;
+  with_modes<Pol>(a.finish, a.comp_mode, [&](auto copy, auto comp) {
+    for (int b = blockIdx.x * kKvWarps + wid; b < T; b += gridDim.x * kKvWarps)
+      kv_tile<Pol, KP, decltype(copy)::value, decltype(comp)::value>(a, b, a.nnz, sm[wid]);
+  });
 }
 
+// a thread per (tile, vector)
 template <class X, int KP>
 __global__ void fixup_spmm(CsrTileView v, const double *head, const double *tail, X *y,
                            int64_t ldy, int k, double alpha, double beta) {
   grid_dependency_wait();
   const int T = v.count();
-  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < T; b += gridDim.x * blockDim.x)
-    fixup_tile_k<X, KP>(v, T, b, head, tail, y, ldy, k, alpha, beta);
+  for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < int64_t(T) * KP;
+       g += int64_t(gridDim.x) * blockDim.x) {
+    const int j = static_cast<int>(g % KP);
+    if (j < k)
+      fixup_tile_k(v, T, static_cast<int>(g / KP), j, KP, head, tail, y, ldy, alpha, beta);
+  }
 }
 
 // resident blocks of a kernel per device (after the dynamic shared-memory
@@ -104,7 +112,9 @@ static size_t spmm_ws_layout(int64_t tiles, int kp, int64_t n, size_t xsize, dou
     char *p = static_cast<char *>(base);
     *head = reinterpret_cast<double *>(p + oh);
     *tail = reinterpret_cast<double *>(p + ot);
-    *xt = p + ox;
+    // the kernels read rows of xt by 32-byte loads; the caller's workspace
+    // is 16-byte aligned (the slack below covers the difference)
+    *xt = reinterpret_cast<void *>((reinterpret_cast<uintptr_t>(p + ox) + 31) & ~uintptr_t(31));
   }
   return o + 256;
 }
@@ -121,12 +131,10 @@ static msrep_status run_spmm(const msrep_matrix *A, const msrep_partition *p, in
   void *xt = nullptr;
   spmm_ws_layout(L.tmax, KP, A->n, sizeof(X), &head, &tail, &xt, ws);
   const int sg = 4 * sm_count();
-  if (A->n > 0) {
-    interleave_x<X, KP><<<sg, 256, 0, st>>>(static_cast<const X *>(x), ldx, k, A->n,
-                                            static_cast<X *>(xt));
-    MSREP_CUDA_TRY(cudaGetLastError());
-  }
-  SpmmArgs<Pol, KP> a;
+  if (A->n > 0)
+    MSREP_TRY(launch_dependent(interleave_x<X, KP>, sg, 256, st, 0, static_cast<const X *>(x),
+                               ldx, k, A->n, static_cast<X *>(xt)));
+  SpmmArgs<Pol> a;
   a.row_ptr = A->ptr;
   a.col_idx = A->idx;
   a.val = static_cast<const typename Pol::V *>(A->val);
@@ -143,20 +151,17 @@ static msrep_status run_spmm(const msrep_matrix *A, const msrep_partition *p, in
   a.tail = tail;
   a.hs = KP;
   a.m = A->m;
+  a.nnz = static_cast<int32_t>(A->nnz);
   a.comp_mode = flags & (MSREP_COMP_ALL | MSREP_COMP_NONE);
   const int32_t *n_tiles = reinterpret_cast<const int32_t *>(plan + L.off_toff) + p->np;
   int nb = 1;
-  // a tile's walk is a chain of dependent loads, so tiles in flight set the
-  // rate: the 1- and 2-vector layouts fit three blocks an SM in registers
-  // (R-MAT FP32, 2 vectors: 207 -> 174 us); the wider ones fit two
-  MSREP_TRY(blocks_of(csr_spmm_direct<Pol, KP>, 0, KP <= 2 ? 3 : 2, &nb));
-  constexpr int G = KvShape<X, KP>::G;
-  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.tmax, G),
+  MSREP_TRY(blocks_of(csr_spmm_direct<Pol, KP>, 0, KvShape<X, KP>::kBlocks, &nb));
+  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.tmax, kKvWarps),
                                                              int64_t(nb) * sm_count()));
-  MSREP_TRY(launch_dependent(csr_spmm_direct<Pol, KP>, grid, kKvThreads, st, 0, a, n_tiles,
-                             A->nnz));
+  MSREP_TRY(launch_dependent(csr_spmm_direct<Pol, KP>, grid, kKvThreads, st, 0, a, n_tiles));
   CsrTileView v{a.tile_row, a.tile_k, A->ptr, n_tiles};
-  const int64_t fg = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.tmax, 256), 4 * sm_count()));
+  const int64_t fg =
+      std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.tmax * KP, 256), 8 * sm_count()));
   MSREP_TRY(launch_dependent(fixup_spmm<X, KP>, fg, 256, st, 0, v,
                              static_cast<const double *>(head), static_cast<const double *>(tail),
                              a.y, ldy, k, alpha, beta));
@@ -192,53 +197,26 @@ __device__ __forceinline__ int owner_item_k(const int64_t *toff, int count, int6
   return lo;
 }
 
-// one block work unit of an item: tile u * G + ts by tile group ts
-template <class Pol, int KP>
-__device__ __forceinline__ void batched_unit(const BatchItem &it, int64_t base, int T, int u,
-                                             const void *xt, void *y, double *head,
-                                             double *tail, unsigned comp_mode,
-                                             KvSmem<typename Pol::Acc, 8> &sm) {
-  using Sh = KvShape<typename Pol::X, KP>;
-  const int ts = threadIdx.x / Sh::GT, b = u * Sh::G + ts;
-  if (b >= T) return;  // uniform over the tile group
-  SpmmArgs<Pol, KP> a;
-  a.row_ptr = it.row_ptr;
-  a.col_idx = it.col_idx;
-  a.val = static_cast<const typename Pol::V *>(it.val);
-  a.xt = static_cast<const typename Pol::X *>(xt);
-  a.y = static_cast<typename Pol::X *>(y);
-  a.ldy = it.m;
-  a.k = it.k;
-  a.alpha = 1.0;
-  a.beta = 0.0;
-  a.finish = kFinishCopy;
-  a.tile_row = it.tile_row;
-  a.tile_k = it.tile_k;
-  a.head = head + base * kBatchWidth;
-  a.tail = tail + base * kBatchWidth;
-  a.hs = kBatchWidth;
-  a.m = it.m;
-  a.comp_mode = comp_mode;
-  kv_tile<Pol, KP, 8>(a, b, it.nnz, sm, ts);
-}
-
 // Items of 2..8 vectors; item j's x interleaved with width KP_j =
 // spmm_width(k_j) and its tiles cut into uoff[j+1] - uoff[j] block work
-// units of KvShape<float, KP_j>::G tiles, one unit per block at a time.
-// Tile groups run ahead of each other within a layout; where the layout
-// (KP) changes from one unit to the next the block synchronises, because
-// the two layouts share shared-memory slots differently.
-template <class Pol>
-__global__ void __launch_bounds__(kKvThreads) batched_spmm(const BatchItem *items,
-                                                           const int64_t *toff,
-                                                           const int64_t *uoff, int count,
-                                                           const void *const *xs,
-                                                           void *const *ys, double *head,
-                                                           double *tail, unsigned comp_mode) {
-  __shared__ KvSmem<typename Pol::Acc, 8> sm;
+// units of kKvWarps tiles, one unit per block at a time, one tile per warp.
+// The warps never wait for one another.
+// The item's pointers are kept in shared memory: in registers they spilled.
+template <class Pol, bool kComp>
+__global__ void __launch_bounds__(kKvThreads, 4)
+    batched_spmm(const BatchItem *items, const int64_t *toff, const int64_t *uoff, int count,
+                 const void *const *xs, void *const *ys, double *head, double *tail) {
+  using X = typename Pol::X;
+  using Slot = KvWarpSmem<X, KvShape<X, 8>::VW>;  // the widest layout's
+  static_assert(sizeof(KvWarpSmem<X, KvShape<X, 2>::VW>) <= sizeof(Slot) &&
+                    sizeof(KvWarpSmem<X, KvShape<X, 4>::VW>) <= sizeof(Slot),
+                "every layout fits the widest one's slot");
+  __shared__ Slot sm[kKvWarps];
+  __shared__ SpmmArgs<Pol> s_args[kKvWarps];
   grid_dependency_wait();
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t total = __ldg(uoff + count);
-  int j = 0, prev_kp = 0;
+  int j = 0, held = -1;
   for (int64_t g = blockIdx.x; g < total; g += gridDim.x) {
     int step = 0;
     while (step < 4 && j + 1 < count && __ldg(uoff + j + 1) <= g) {
@@ -246,45 +224,74 @@ __global__ void __launch_bounds__(kKvThreads) batched_spmm(const BatchItem *item
       ++step;
     }
     if (step == 4) j = owner_item_k(uoff, count, g);
-    const BatchItem it = items[j];
     const int64_t base = __ldg(toff + j);
     const int T = static_cast<int>(__ldg(toff + j + 1) - base);
-    const int u = static_cast<int>(g - __ldg(uoff + j));
-    const int kp = spmm_width(it.k);
-    if (kp != prev_kp) {
-      __syncthreads();
-      prev_kp = kp;
+    const int b = static_cast<int>(g - __ldg(uoff + j)) * kKvWarps + wid;
+    if (b >= T) continue;  // warp-uniform
+    SpmmArgs<Pol> &a = s_args[wid];
+    if (j != held) {
+      held = j;
+      __syncwarp();
+      if (lane == 0) {
+        const BatchItem it = items[j];
+        a.row_ptr = it.row_ptr;
+        a.col_idx = it.col_idx;
+        a.val = static_cast<const typename Pol::V *>(it.val);
+        a.xt = static_cast<const X *>(xs[j]);
+        a.y = static_cast<X *>(ys[j]);
+        a.ldy = it.m;
+        a.k = it.k;
+        a.alpha = 1.0;
+        a.beta = 0.0;
+        a.finish = kFinishCopy;
+        a.tile_row = it.tile_row;
+        a.tile_k = it.tile_k;
+        a.head = head + base * kBatchWidth;
+        a.tail = tail + base * kBatchWidth;
+        a.hs = kBatchWidth;
+        a.m = it.m;
+        a.nnz = static_cast<int32_t>(it.nnz);
+      }
+      __syncwarp();
     }
+    const int kp = spmm_width(a.k);
     if (kp == 2)
-      batched_unit<Pol, 2>(it, base, T, u, xs[j], ys[j], head, tail, comp_mode, sm);
+      kv_tile<Pol, 2, true, kComp>(
+          a, b, a.nnz, *reinterpret_cast<KvWarpSmem<X, KvShape<X, 2>::VW> *>(sm + wid));
     else if (kp == 4)
-      batched_unit<Pol, 4>(it, base, T, u, xs[j], ys[j], head, tail, comp_mode, sm);
+      kv_tile<Pol, 4, true, kComp>(
+          a, b, a.nnz, *reinterpret_cast<KvWarpSmem<X, KvShape<X, 4>::VW> *>(sm + wid));
     else
-      batched_unit<Pol, 8>(it, base, T, u, xs[j], ys[j], head, tail, comp_mode, sm);
+      kv_tile<Pol, 8, true, kComp>(a, b, a.nnz, sm[wid]);
   }
 }
 
+// a thread per (tile, vector)
 template <class X>
 __global__ void batched_fixup_k(const BatchItem *items, const int64_t *toff, int count,
                                 void *const *ys, const double *head, const double *tail) {
   grid_dependency_wait();
   constexpr int KP = kBatchWidth;
-  const int64_t total = __ldg(toff + count);
+  const int64_t total = __ldg(toff + count) * KP;
   for (int64_t g = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; g < total;
        g += int64_t(gridDim.x) * blockDim.x) {
-    const int j = owner_item_k(toff, count, g);
+    const int64_t t = g / KP;
+    const int v = static_cast<int>(g % KP);
+    const int j = owner_item_k(toff, count, t);
     const int64_t base = __ldg(toff + j);
     const int T = static_cast<int>(__ldg(toff + j + 1) - base);
     const BatchItem it = items[j];
+    if (v >= it.k) continue;
     struct View {
       const int32_t *tile_row, *tile_k, *row_ptr;
       __device__ void row_flag(int b, int32_t &r, bool &f) const {
         r = __ldg(tile_row + b);
         f = __ldg(row_ptr + r) < __ldg(tile_k + b);
       }
-    } v{it.tile_row, it.tile_k, it.row_ptr};
-    fixup_tile_k<X, KP>(v, T, static_cast<int>(g - base), head + base * KP, tail + base * KP,
-                        static_cast<X *>(ys[j]), it.m, it.k, 1.0, 0.0);
+      __device__ bool continues(int b, int32_t r) const { return __ldg(tile_row + b) == r; }
+    } view{it.tile_row, it.tile_k, it.row_ptr};
+    fixup_tile_k(view, T, static_cast<int>(t - base), v, KP, head + base * KP, tail + base * KP,
+                 static_cast<X *>(ys[j]), it.m, 1.0, 0.0);
   }
 }
 
@@ -310,12 +317,7 @@ __global__ void interleave_batch(const BatchItem *items, int count, const void *
   }
 }
 
-int64_t batched_k_units(int64_t tiles, int k) {
-  const int kp = spmm_width(k);
-  const int g = kp == 2 ? KvShape<float, 2>::G : kp == 4 ? KvShape<float, 4>::G
-                                                         : KvShape<float, 8>::G;
-  return (tiles + g - 1) / g;
-}
+int64_t batched_k_units(int64_t tiles, int) { return (tiles + kKvWarps - 1) / kKvWarps; }
 
 msrep_status launch_batched_k(const BatchItem *items, const int64_t *toff, const int64_t *uoff,
                               int count, int64_t total_tiles, int64_t total_units,
@@ -326,14 +328,16 @@ msrep_status launch_batched_k(const BatchItem *items, const int64_t *toff, const
   interleave_batch<float><<<dim3(64, std::min(count, 1024)), 256, 0, st>>>(items, count, xin, xt);
   MSREP_CUDA_TRY(cudaGetLastError());
   if (total_tiles == 0) return MSREP_OK;
-  const unsigned comp = flags & (MSREP_COMP_ALL | MSREP_COMP_NONE);
+  const auto kern = (flags & (MSREP_COMP_ALL | MSREP_COMP_NONE)) == MSREP_COMP_NONE
+                        ? batched_spmm<PolF32<float>, false>
+                        : batched_spmm<PolF32<float>, true>;
   int nb = 1;
-  MSREP_TRY(blocks_of(batched_spmm<PolF32<float>>, 0, 2, &nb));
+  MSREP_TRY(blocks_of(kern, 0, 4, &nb));
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(total_units, int64_t(nb) * sms));
-  MSREP_TRY(launch_dependent(batched_spmm<PolF32<float>>, grid, kKvThreads, st, 0, items, toff,
-                             uoff, count, static_cast<const void *const *>(xt), ys, head, tail,
-                             comp));
-  const int64_t fg = std::max<int64_t>(1, std::min<int64_t>(ceil_div(total_tiles, 256), 4 * sms));
+  MSREP_TRY(launch_dependent(kern, grid, kKvThreads, st, 0, items, toff, uoff, count,
+                             static_cast<const void *const *>(xt), ys, head, tail));
+  const int64_t fg = std::max<int64_t>(
+      1, std::min<int64_t>(ceil_div(total_tiles * kBatchWidth, 256), 8 * sms));
   MSREP_TRY(launch_dependent(batched_fixup_k<float>, fg, 256, st, 0, items, toff, count, ys,
                              static_cast<const double *>(head), static_cast<const double *>(tail)));
   return MSREP_OK;

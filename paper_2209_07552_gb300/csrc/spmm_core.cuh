@@ -5,31 +5,41 @@
 // nonzero gathers one contiguous 4..64-byte segment, and the matrix is
 // streamed once for all k vectors.
 //
-// Thread layout: TPV threads share lane vl of a tile, each holding VPT =
-// KP / TPV of the vectors (one vector load of its part of the x row per
-// nonzero).  A block of 256 threads holds G = 8 / TPV tile groups of 32 *
-// TPV threads, each walking its own tiles and synchronising only with
-// itself.
-// Each thread walks exactly the nonzeros that lane vl of the SpMV's warp
-// walks, with the same FMAs in the same order for each of its vectors
-// (masked positions included), and finishes the same rows; the SpMV's warp
-// segmented scan then runs once per (tile, vector) on the lane partials,
-// gathered through shared memory.  So Y[:, v] equals msrep_spmv of x_v bit
-// for bit.  TPV is kept small (VPT up to 4 FP32 or 2 FP64 values) so that a
-// block holds many tiles: the tile walk is a chain of dependent memory
-// round trips, and tiles in flight set the throughput.
+// One warp works on a tile alone, lane l walking exactly the nonzeros that
+// lane l of the SpMV's warp walks, with the same FMAs in the same order for
+// each vector (masked positions add zero) and the same warp scan, so
+// Y[:, v] equals msrep_spmv of x_v bit for bit.  A lane holds VW vectors: up
+// to 32 bytes of an x row, fetched by one 256-bit load (FP64 with eight
+// vectors takes two passes over the tile).
+//
+// What bounds it: one L1 line lookup per nonzero for the gather (16.8M of
+// them take about 55 us on 152 SMs) and, above that, the instructions around
+// it at 16 warps an SM (87M warp instructions on the R-MAT matrix, k = 8;
+// issue slots 46% used, L1 60%).  Measured on R-MAT 2^20 / 2^24 nonzeros,
+// FP32, the whole call: k = 2 / 4 / 8 113 / 136 / 207 us, against 186 / 345 /
+// 539 us with row ends walked inside the nonzero loop and y written from
+// there (197M warp instructions at k = 8); 2048^2 Laplacian k = 8 302 against
+// 481 us.  Three things keep the instructions few:
+//  * where the rows of the tile end is worked out once per tile, a lane per
+//    row, into a bit string in shared memory; the nonzero loop tests one bit
+//    instead of walking row pointers on a divergent path;
+//  * a finished row is stored into a row buffer in shared memory, and y is
+//    written a lane per row afterwards (consecutive rows of one vector in one
+//    store), instead of KP scattered stores per row end;
+//  * FP32 arithmetic runs on pairs of vectors (the packed f32x2
+//    instructions, each half rounded as the scalar instruction).
 #pragma once
 
 #include "spmv_core.cuh"
 
 namespace msrep {
 
-template <class Pol, int KP>
+template <class Pol>
 struct SpmmArgs {
   const int32_t *row_ptr;
   const int32_t *col_idx;
   const typename Pol::V *val;
-  const typename Pol::X *xt;  // [n][KP] interleaved
+  const typename Pol::X *xt;  // [n][KP] interleaved, 32-byte aligned
   typename Pol::X *y;         // y[v * ldy + row], v < k
   int64_t ldy;
   int k;
@@ -39,6 +49,7 @@ struct SpmmArgs {
   double *head, *tail;  // [T][hs]: tile b's partial of vector v at b * hs + v
   int hs;               // head / tail stride (>= KP)
   int32_t m;
+  int32_t nnz;
   unsigned comp_mode;
 };
 
@@ -47,259 +58,553 @@ __host__ __device__ constexpr int spmm_width(int k) {
   return k <= 1 ? 1 : k <= 2 ? 2 : k <= 4 ? 4 : 8;
 }
 
-// threads per lane: at most 4 FP32 (16 bytes) or 2 FP64 x values a thread
+// vectors a lane holds at once: as many as fit a 32-byte load
 template <class X, int KP>
 struct KvShape {
-  static constexpr int VMAX = sizeof(X) == 8 ? 2 : 4;
-  static constexpr int TPV = KP > VMAX ? KP / VMAX : 1;
-  static constexpr int VPT = KP / TPV;
-  static constexpr int G = 8 / TPV;  // tile groups of a 256-thread block
-  static constexpr int GT = 32 * TPV;  // threads of a tile group
+  static constexpr int VW = KP * int(sizeof(X)) <= 32 ? KP : 32 / int(sizeof(X));
+  // Resident blocks (of 4 warps) per SM asked of the register allocator: 32
+  // bytes of x a lane need about 120 registers, and five blocks (96, with
+  // spills) took 215 us where four take 207 (R-MAT, FP32, k = 8); the
+  // narrower ones fit more.
+  static constexpr int kBlocks = VW * int(sizeof(X)) == 32 ? 4 : VW * int(sizeof(X)) == 16 ? 6 : 7;
 };
 
-constexpr int kKvWarps = 8;
+constexpr int kKvWarps = 4;
 constexpr int kKvThreads = 32 * kKvWarps;
-constexpr int kKvRowSlots = 32 * 32 + 8;  // row pointers of a tile of <= 1024
+constexpr int kKvBitWords = 34;   // a tile of <= 1024 nonzeros in aligned groups of 8
+constexpr int kKvRows = 88;       // rows of the row buffer
 
-// Shared memory of a block: the row pointers of its GS tile groups, the
-// lane partials of the scans (four rows of 33 per warp, [vector][lane],
-// 33 against bank conflicts) and the lanes' row-finished flags.
-template <class Acc, int GS>
-struct KvSmem {
-  int32_t rp[GS][kKvRowSlots];
-  Acc part[32 * 33];
-  int32_t flag[GS * 32];
+// Shared memory of one warp.  A stored accumulator is VW sums, then (FP32)
+// their VW compensations; 16 bytes of padding from 32 bytes on let a warp
+// read one per lane without bank conflicts.
+template <class X, int VW>
+struct KvWarpSmem {
+  static constexpr int kAcc = (sizeof(X) == 4 ? 2 : 1) * VW;
+  static constexpr int kSlot = kAcc * int(sizeof(X)) >= 32 ? kAcc + 16 / int(sizeof(X)) : kAcc;
+  // finished rows' accumulators in the order of the rows' ends.  kKvRows
+  // holds every tile of 512 whose rows average five nonzeros; a tile with
+  // more row ends is walked once for each kKvRows of them.
+  alignas(16) X rows[kKvRows][kSlot];
+  alignas(16) X last[kAcc];          // the row that continues past the tile
+  uint32_t end[kKvBitWords];         // bit e: a row ends with element e of the tile
 };
 
-// VPT consecutive x values (16-byte vector loads where they fit)
-template <int VPT>
-__device__ __forceinline__ void ldx(const float *p, float (&o)[VPT]) {
-  if constexpr (VPT == 1) {
-    o[0] = __ldg(p);
-  } else if constexpr (VPT == 2) {
-    const float2 t = __ldg(reinterpret_cast<const float2 *>(p));
-    o[0] = t.x;
-    o[1] = t.y;
+// Vector j of a stored accumulator as the FP64 partial of a split row.
+template <int VW>
+__device__ __forceinline__ double kv_partial(const double *p, int j) { return p[j]; }
+template <int VW>
+__device__ __forceinline__ double kv_partial(const float *p, int j) {
+  return pair_total_f64(p[j], p[VW + j]);
+}
+
+// ---------------------------------------------------------------------------
+// VW vectors' accumulators and x values of one lane
+// ---------------------------------------------------------------------------
+
+using f32x2 = unsigned long long;  // two binary32 values, the lower lane first
+
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &a, float &b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+template <class Pol, int VW>
+struct KvAcc;
+
+// FP64: VW sums.
+template <int VW>
+struct KvAcc<PolF64, VW> {
+  using X = double;
+  double a[VW];
+  struct XV {
+    double d[VW];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+      for (int j = 0; j < VW; ++j) d[j] = 0.0;
+    }
+    __device__ __forceinline__ void load(const double *p) {
+      if constexpr (VW == 1) {
+        d[0] = __ldg(p);
+      } else if constexpr (VW == 2) {
+        const double2 t = __ldg(reinterpret_cast<const double2 *>(p));
+        d[0] = t.x;
+        d[1] = t.y;
+      } else {
+        static_assert(VW == 4, "32-byte loads");
+        asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+            : "=d"(d[0]), "=d"(d[1]), "=d"(d[2]), "=d"(d[3])
+            : "l"(p));
+      }
+    }
+  };
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int j = 0; j < VW; ++j) a[j] = 0.0;
+  }
+  template <bool kComp>
+  __device__ __forceinline__ void fma(double v, const XV &x) {
+#pragma unroll
+    for (int j = 0; j < VW; ++j) a[j] = __fma_rn(v, x.d[j], a[j]);
+  }
+  __device__ __forceinline__ void store(double *p) const {
+    if constexpr (VW == 1) {
+      p[0] = a[0];
+    } else {
+#pragma unroll
+      for (int j = 0; j < VW; j += 2)
+        *reinterpret_cast<double2 *>(p + j) = make_double2(a[j], a[j + 1]);
+    }
+  }
+  __device__ __forceinline__ void load(const double *p) {
+    if constexpr (VW == 1) {
+      a[0] = p[0];
+    } else {
+#pragma unroll
+      for (int j = 0; j < VW; j += 2) {
+        const double2 t = *reinterpret_cast<const double2 *>(p + j);
+        a[j] = t.x;
+        a[j + 1] = t.y;
+      }
+    }
+  }
+  __device__ __forceinline__ void totals(double (&t)[VW]) const {
+#pragma unroll
+    for (int j = 0; j < VW; ++j) t[j] = a[j];
+  }
+  // *this = u + *this
+  __device__ __forceinline__ void carry_in(const KvAcc &u) {
+#pragma unroll
+    for (int j = 0; j < VW; ++j) a[j] = __dadd_rn(u.a[j], a[j]);
+  }
+  __device__ __forceinline__ KvAcc shfl_up(int o) const {
+    KvAcc r;
+#pragma unroll
+    for (int j = 0; j < VW; ++j) r.a[j] = __shfl_up_sync(0xffffffffu, a[j], o);
+    return r;
+  }
+};
+
+// FP32 sums and their compensation, two vectors to a register pair.  The
+// compensated update is PolF32::fma's on each half; the product is formed
+// negated (n = -v x, exactly the negative of v x rounded), which turns its
+// uses into subtractions and leaves every rounding as it was.
+template <class VT, int VW>
+struct KvAcc<PolF32<VT>, VW> {
+  using X = float;
+  static constexpr int N2 = VW / 2;
+  f32x2 s[N2], c[N2];
+  struct XV {
+    f32x2 d[N2];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+      for (int j = 0; j < N2; ++j) d[j] = 0;
+    }
+    __device__ __forceinline__ void load(const float *p) {
+      if constexpr (VW == 2) {
+        asm("ld.global.nc.b64 %0, [%1];" : "=l"(d[0]) : "l"(p));
+      } else if constexpr (VW == 4) {
+        asm("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(d[0]), "=l"(d[1]) : "l"(p));
+      } else {
+        static_assert(VW == 8, "32-byte loads");
+        asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];"
+            : "=l"(d[0]), "=l"(d[1]), "=l"(d[2]), "=l"(d[3])
+            : "l"(p));
+      }
+    }
+  };
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int j = 0; j < N2; ++j) s[j] = c[j] = 0;
+  }
+  template <bool kComp>
+  __device__ __forceinline__ void fma(float v, const XV &x) {
+    const f32x2 vv = pack2(v, v);
+    if (kComp) {
+      const f32x2 nv = pack2(-v, -v);
+#pragma unroll
+      for (int j = 0; j < N2; ++j) {
+        const f32x2 n = mul2(nv, x.d[j]);            // -p
+        const f32x2 ep = fma2(vv, x.d[j], n);        // v x - p
+        const f32x2 t = sub2(s[j], n);               // s + p
+        const f32x2 bb = sub2(t, s[j]), aa = sub2(t, bb);
+        const f32x2 es = sub2(sub2(s[j], aa), add2(n, bb));
+        s[j] = t;
+        c[j] = add2(c[j], add2(ep, es));
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < N2; ++j) s[j] = fma2(vv, x.d[j], s[j]);
+    }
+  }
+  __device__ __forceinline__ void store(float *p) const {
+    ulonglong2 *q = reinterpret_cast<ulonglong2 *>(p);  // 16-byte accesses
+    if constexpr (N2 == 1) {
+      q[0] = make_ulonglong2(s[0], c[0]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < N2 / 2; ++j) {
+        q[j] = make_ulonglong2(s[2 * j], s[2 * j + 1]);
+        q[N2 / 2 + j] = make_ulonglong2(c[2 * j], c[2 * j + 1]);
+      }
+    }
+  }
+  __device__ __forceinline__ void load(const float *p) {
+    const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(p);
+    if constexpr (N2 == 1) {
+      const ulonglong2 t = q[0];
+      s[0] = t.x;
+      c[0] = t.y;
+    } else {
+#pragma unroll
+      for (int j = 0; j < N2 / 2; ++j) {
+        const ulonglong2 t = q[j], w = q[N2 / 2 + j];
+        s[2 * j] = t.x;
+        s[2 * j + 1] = t.y;
+        c[2 * j] = w.x;
+        c[2 * j + 1] = w.y;
+      }
+    }
+  }
+  __device__ __forceinline__ void totals(float (&t)[VW]) const {
+#pragma unroll
+    for (int j = 0; j < N2; ++j) {
+      float s0, s1, c0, c1;
+      unpack2(s[j], s0, s1);
+      unpack2(c[j], c0, c1);
+      t[2 * j] = pair_total(s0, c0);
+      t[2 * j + 1] = pair_total(s1, c1);
+    }
+  }
+  __device__ __forceinline__ void carry_in(const KvAcc &u) {
+#pragma unroll
+    for (int j = 0; j < N2; ++j) {
+      const f32x2 t = add2(u.s[j], s[j]);
+      const f32x2 bb = sub2(t, u.s[j]), aa = sub2(t, bb);
+      const f32x2 e = add2(sub2(u.s[j], aa), sub2(s[j], bb));
+      s[j] = t;
+      c[j] = add2(add2(u.c[j], c[j]), e);
+    }
+  }
+  __device__ __forceinline__ KvAcc shfl_up(int o) const {
+    KvAcc r;
+#pragma unroll
+    for (int j = 0; j < N2; ++j) {
+      r.s[j] = __shfl_up_sync(0xffffffffu, s[j], o);
+      r.c[j] = __shfl_up_sync(0xffffffffu, c[j], o);
+    }
+    return r;
+  }
+};
+
+// one FP32 vector
+template <class VT>
+struct KvAcc<PolF32<VT>, 1> {
+  using X = float;
+  using Pol = PolF32<VT>;
+  F32Pair a;
+  struct XV {
+    float d;
+    __device__ __forceinline__ void zero() { d = 0.f; }
+    __device__ __forceinline__ void load(const float *p) { d = __ldg(p); }
+  };
+  __device__ __forceinline__ void zero() { a = Pol::zero(); }
+  template <bool kComp>
+  __device__ __forceinline__ void fma(float v, const XV &x) {
+    a = Pol::template fma<kComp>(a, v, x.d);
+  }
+  __device__ __forceinline__ void store(float *p) const {
+    p[0] = a.s;
+    p[1] = a.c;
+  }
+  __device__ __forceinline__ void load(const float *p) { a = F32Pair{p[0], p[1]}; }
+  __device__ __forceinline__ void totals(float (&t)[1]) const { t[0] = pair_total(a.s, a.c); }
+  __device__ __forceinline__ void carry_in(const KvAcc &u) { a = Pol::combine(u.a, a); }
+  __device__ __forceinline__ KvAcc shfl_up(int o) const {
+    KvAcc r;
+    r.a = Pol::shfl_up(a, o);
+    return r;
+  }
+};
+
+// y of a finished row from its total t (s + c of the low-precision form),
+// rounded as Pol::finish rounds it
+__device__ __forceinline__ double finish_total(double t, int mode, double alpha, double beta,
+                                               const double *y) {
+  return PolF64::finish(t, mode, alpha, beta, y);
+}
+__device__ __forceinline__ float finish_total(float t, int mode, double alpha, double beta,
+                                              const float *y) {
+  if (mode == kFinishCopy) return t;
+  const float r = __fmul_rn(float(alpha), t);
+  if (mode == kFinishScale) return r;
+  return __fmaf_rn(float(beta), *y, r);
+}
+
+// Four consecutive elements at h4 (a multiple of 4): one vector load, or
+// element-wise at the array's end.
+__device__ __forceinline__ void ld4(const int32_t *p, int32_t (&r)[4]) {
+  asm("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+      : "l"(p));
+}
+__device__ __forceinline__ void ld4(const float *p, float (&r)[4]) {
+  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3])
+      : "l"(p));
+}
+__device__ __forceinline__ void ld4(const double *p, double (&r)[4]) {
+  asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];"
+      : "=d"(r[0]), "=d"(r[1]), "=d"(r[2]), "=d"(r[3])
+      : "l"(p));
+}
+__device__ __forceinline__ void ld4(const bf16_t *p, float (&r)[4]) {
+  uint32_t w[2];
+  asm("ld.global.nc.L1::no_allocate.v2.b32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    r[2 * i] = __uint_as_float(w[i] << 16);
+    r[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
+template <class T, class U>
+__device__ __forceinline__ void load4(const T *arr, int32_t h4, int32_t nnz, U (&out)[4]) {
+  if (h4 < (nnz & ~3)) {
+    ld4(arr + h4, out);
   } else {
-    const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
-    o[0] = t.x;
-    o[1] = t.y;
-    o[2] = t.z;
-    o[3] = t.w;
-  }
-}
-template <int VPT>
-__device__ __forceinline__ void ldx(const double *p, double (&o)[VPT]) {
-  if constexpr (VPT == 1) {
-    o[0] = __ldg(p);
-  } else {
-    const double2 t = __ldg(reinterpret_cast<const double2 *>(p));
-    o[0] = t.x;
-    o[1] = t.y;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) out[u] = (u < nnz - h4) ? U(ld_stream(arr + h4 + u)) : U(0);
   }
 }
 
-// kCopy: alpha = 1, beta = 0 known at compile time (the copy finish)
-template <class Pol, int KP, bool kCopy = false>
-__device__ __forceinline__ void spmm_write_row(const SpmmArgs<Pol, KP> &a, int v, int32_t row,
-                                               typename Pol::Acc acc) {
-  if (v < a.k) {
-    typename Pol::X *yp = a.y + v * a.ldy + row;
-    *yp = Pol::finish(acc, kCopy ? int(kFinishCopy) : a.finish, a.alpha, a.beta, yp);
-  }
-}
-
-// Synchronise the GT threads of tile group ts (a warp, or a named barrier
-// over the group's warps).
-template <int GT>
-__device__ __forceinline__ void group_sync(int ts) {
-  if constexpr (GT == 32)
-    __syncwarp();
-  else
-    asm volatile("bar.sync %0, %1;" ::"r"(ts + 1), "n"(GT) : "memory");
-}
-
-// Tile b by tile group ts (threads ts*GT .. ts*GT+GT-1 of the block; all
-// of them call it).  Shared memory used: rp[ts] and the partial rows
-// ts*TPV*4 .. ts*TPV*4 + KP - 1, so groups never touch each other's
-// slots and synchronise only among themselves.
-template <class Pol, int KP, int GS, bool kCopy = false>
-__device__ __forceinline__ void kv_tile(const SpmmArgs<Pol, KP> &a, int b, int64_t nnz,
-                                        KvSmem<typename Pol::Acc, GS> &sm, int ts) {
-  using Acc = typename Pol::Acc;
-  using LV = typename LoadT<typename Pol::V>::type;
+// Tile b by one warp.  kCopy: alpha = 1, beta = 0 known at compile time;
+// kComp: compensated sums (low-precision form).
+template <class Pol, int KP, bool kCopy, bool kComp>
+__device__ __forceinline__ void kv_tile(const SpmmArgs<Pol> &a, int b, int32_t nnz,
+                                        KvWarpSmem<typename Pol::X, KvShape<typename Pol::X, KP>::VW> &sm) {
   using X = typename Pol::X;
-  using Sh = KvShape<X, KP>;
-  constexpr int TPV = Sh::TPV, VPT = Sh::VPT, GT = 32 * TPV;
-  static_assert(GS >= Sh::G, "too few row-pointer slots");
-  const int q = threadIdx.x % GT, vl = q / TPV, v0 = (q % TPV) * VPT;
-  const int prow = ts * TPV * 4;  // first partial row of the group
-  int32_t *rp = sm.rp[ts];
+  using LV = typename LoadT<typename Pol::V>::type;
+  constexpr int VW = KvShape<X, KP>::VW;
+  using Acc = KvAcc<Pol, VW>;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int fin = kCopy ? int(kFinishCopy) : a.finish;
   const int32_t r0 = __ldg(a.tile_row + b), k0 = __ldg(a.tile_k + b);
   const int32_t r1 = __ldg(a.tile_row + b + 1), k1 = __ldg(a.tile_k + b + 1);
-  {
-    const int32_t rend = min(r1 + 2, a.m + 1);
-    for (int32_t r = r0 + q; r < rend; r += GT) rp[r - r0] = __ldg(a.row_ptr + r);
-  }
-  group_sync<GT>(ts);
-
-  // lane vl of csr_tile_compute, for vectors v0 .. v0 + VPT - 1
-  Acc acc[VPT], first_acc[VPT];
-#pragma unroll
-  for (int j = 0; j < VPT; ++j) acc[j] = first_acc[j] = Pol::zero();
-  bool emitted = false;
-  int first_r = 0;
   const int nrows = r1 - r0;
-  const int32_t rs0 = rp[0];
-  const int32_t *s_end = rp + 1;
-  const bool flag = rs0 < k0;
-  {
-    const LaneRange lr = lane_range(k0, k1, vl);
-    const int32_t ka = static_cast<int32_t>(lr.ka), kb = static_cast<int32_t>(lr.kb);
-    int r = vl == 0 ? 0 : upper_bound_smem(s_end, nrows, ka);
-    const int r_end = upper_bound_smem(s_end, nrows, kb);
-    int32_t next_end = r < r_end ? s_end[r] : INT32_MAX;
-    int32_t re_last = 0;
-    if (Pol::kLow) re_last = (r1 < a.m) ? rp[nrows + 1] : k1;
-    auto row_comp = [&](int rr) -> bool {
-      if (!Pol::kLow) return false;
-      int64_t st = rr == 0 ? int64_t(rs0) : int64_t(s_end[rr - 1]);
-      int64_t en = rr < nrows ? int64_t(s_end[rr]) : int64_t(re_last);
-      return want_comp(a.comp_mode, en - st, (rr == 0 && flag) || rr == nrows);
-    };
-    bool comp = row_comp(r);
-    auto finish_rows = [&](int32_t kk) {
-      while (next_end <= kk) {
-        if (!emitted) {
-          emitted = true;
-          first_r = r;
-#pragma unroll
-          for (int j = 0; j < VPT; ++j) first_acc[j] = acc[j];
-        } else {
-#pragma unroll
-          for (int j = 0; j < VPT; ++j) spmm_write_row<Pol, KP, kCopy>(a, v0 + j, r0 + r, acc[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < VPT; ++j) acc[j] = Pol::zero();
-        ++r;
-        next_end = r < r_end ? s_end[r] : INT32_MAX;
-        comp = row_comp(r);
-      }
-    };
-    finish_rows(ka);
-    const X *xv_base = a.xt + v0;
-    for (int64_t g = lr.glo; g < lr.ghi; ++g) {
-      const int64_t g8 = g << 3;
-      int32_t c[8];
-      LV vv[8];
-      X xv[8][VPT];
-      load_group(a.col_idx, g8, nnz, c);
-      load_group(a.val, g8, nnz, vv);
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const bool in = g8 + u >= ka && g8 + u < kb;
-        if (in) {
-          ldx<VPT>(xv_base + int64_t(c[u]) * KP, xv[u]);
-        } else {
-#pragma unroll
-          for (int j = 0; j < VPT; ++j) xv[u][j] = X(0);
-          vv[u] = LV(0);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        // a branch, not a select: the compensated update is about ten
-        // instructions a vector and rows that need it are few
-        if (Pol::kLow && comp) {
-#pragma unroll
-          for (int j = 0; j < VPT; ++j) acc[j] = Pol::fma(acc[j], vv[u], xv[u][j], true);
-        } else {
-#pragma unroll
-          for (int j = 0; j < VPT; ++j) acc[j] = Pol::fma(acc[j], vv[u], xv[u][j], false);
-        }
-        const int32_t kk = static_cast<int32_t>(g8 + u + 1);
-        if (next_end <= kk) finish_rows(kk);
-      }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < VPT; ++j) sm.part[(prow + v0 + j) * 33 + vl] = acc[j];
-  if (v0 == 0) sm.flag[ts * 32 + vl] = emitted;
-  group_sync<GT>(ts);
+  const int32_t base = k0 & ~7;  // element e of the tile is nonzero base + e
+  const LaneRange lr = lane_range(k0, k1, lane);
+  const int h_lo = static_cast<int>(lr.glo) * 2, h_hi = static_cast<int>(lr.ghi) * 2;
 
-  // the group's warps scan its KP vectors (warp wg: vectors wg*VPT ..),
-  // each as warp_seg_scan does for the SpMV's warp
+  // the lane's first nonzeros, in flight while the rows are worked out
+  int32_t cn[4];
+  LV vn[4];
+  if (h_lo < h_hi) {
+    load4(a.col_idx, h_lo * 4, nnz, cn);
+    load4(a.val, h_lo * 4, nnz, vn);
+  }
+
+  // --- the tile's rows: row i (a lane each) ends in the tile for i < nrows;
+  // row nrows, if the matrix has it, continues past it
+  for (int i = lane; i < kKvBitWords; i += 32) sm.end[i] = 0;
+  __syncwarp();
+  bool flag = false, has0 = false;  // row 0: started earlier; holds a nonzero of the tile
+  int32_t last_end = 0;             // row_ptr[r1]
+  int ends = 0;                     // rows that hold a nonzero of the tile and end in it
+  for (int i0 = 0; i0 <= nrows; i0 += 32) {
+    const int i = i0 + lane;
+    const bool valid = i <= nrows;
+    const int32_t st = valid ? __ldg(a.row_ptr + r0 + i) : 0;
+    const int32_t en = valid && r0 + i < a.m ? __ldg(a.row_ptr + r0 + i + 1) : k1;
+    const int32_t from = max(st, k0), to = min(en, k1);
+    const bool holds = valid && to > from;
+    const bool done = holds && i < nrows;
+    const unsigned dm = __ballot_sync(full, done);
+    if (i0 == 0) {
+      flag = __shfl_sync(full, st, 0) < k0;
+      has0 = (dm & 1u) != 0;
+    }
+    if (done) atomicOr(sm.end + ((to - 1 - base) >> 5), 1u << ((to - 1 - base) & 31));
+    if (nrows - i0 < 32) last_end = __shfl_sync(full, st, nrows - i0);
+    ends += __popc(dm);
+  }
+  __syncwarp();
+
+  // rank of the lane's first row end among the tile's
+  const int gA = k0 >> 3;
+  int rank0;
   {
-    const int lane = threadIdx.x & 31, wg = q >> 5;
-    const bool f = sm.flag[ts * 32 + lane] != 0;
+    int cnt = 0;
+    for (int g = static_cast<int>(lr.glo) - gA; g < static_cast<int>(lr.ghi) - gA; ++g)
+      cnt += __popc((sm.end[g >> 2] >> ((g & 3) * 8)) & 0xffu);
+    int inc = cnt;
 #pragma unroll
-    for (int j = 0; j < VPT; ++j) {
-      const int vw = wg * VPT + j, idx = (prow + vw) * 33 + lane;
-      Acc last;
-      const Acc ex = warp_seg_scan<Pol>(f, sm.part[idx], last);
-      sm.part[idx] = ex;
-      if (lane == 31) {
-        double *dst = nullptr;
-        if (nrows == 0) {
-          if (flag)
-            dst = a.head;
-          else if (k1 > k0)
-            dst = a.tail;
-        } else if (k1 > rp[nrows]) {
-          dst = a.tail;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(full, inc, o);
+      if (lane >= o) inc += t;
+    }
+    rank0 = inc - cnt;
+  }
+
+  // rows [w0, w0 + kKvRows) of the row ends, vectors [v0, v0 + VW)
+  for (int w0 = 0, v0 = 0; v0 < KP;) {
+    // --- the lane's nonzeros
+    const X *xb = a.xt + v0;
+    Acc acc;
+    acc.zero();
+    int rank = rank0 - w0;
+    if ((v0 > 0 || w0 > 0) && h_lo < h_hi) {
+      load4(a.col_idx, h_lo * 4, nnz, cn);
+      load4(a.val, h_lo * 4, nnz, vn);
+    }
+    for (int h = h_lo; h < h_hi; ++h) {
+      const int32_t h4 = h * 4;
+      const int e = h4 - base;
+      // which of the four are the tile's, and end a row
+      const int lo = max(k0 - h4, 0), hi = min(k1 - h4, 4);
+      const uint32_t in = hi > lo ? (0xfu >> (4 - (hi - lo))) << lo : 0u;
+      const uint32_t eb = sm.end[e >> 5] >> (e & 31);
+      LV v[4];
+      typename Acc::XV x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        v[u] = vn[u];
+        if ((in >> u) & 1u) x[u].load(xb + int64_t(cn[u]) * KP);
+      }
+      if (h + 1 < h_hi) {
+        load4(a.col_idx, h4 + 4, nnz, cn);
+        load4(a.val, h4 + 4, nnz, vn);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if ((in >> u) & 1u) acc.template fma<kComp>(v[u], x[u]);
+        if ((eb >> u) & 1u) {  // a row ends here
+          if (static_cast<unsigned>(rank) < unsigned(kKvRows)) acc.store(sm.rows[rank]);
+          ++rank;
+          acc.zero();
         }
-        if (dst) dst[int64_t(b) * a.hs + vw] = Pol::to_f64(last);
       }
     }
-  }
-  group_sync<GT>(ts);
-  if (emitted) {
+
+    // --- rows split between lanes: warp_seg_scan's doubling, for all VW
+    const bool emitted = rank > rank0 - w0;
+    bool f = emitted;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+      if (__all_sync(full, f || lane < o)) break;
+      const Acc u = acc.shfl_up(o);
+      const int fu = __shfl_up_sync(full, int(f), o);
+      if (lane >= o) {
+        if (!f) acc.carry_in(u);
+        f = f || fu;
+      }
+    }
+    Acc ex = acc.shfl_up(1);
+    if (lane == 0) ex.zero();
+    if (emitted && static_cast<unsigned>(rank0 - w0) < unsigned(kKvRows)) {
+      Acc tot;
+      tot.load(sm.rows[rank0 - w0]);
+      tot.carry_in(ex);
+      tot.store(sm.rows[rank0 - w0]);
+    }
+    if (lane == 31) acc.store(sm.last);
+    __syncwarp();
+
+    // --- partials of the rows split between tiles, widened to FP64 a lane
+    // per vector (an FP64 warp instruction costs its full slot of the FP64
+    // pipe however few lanes it has): lanes 0.. the first row's, lanes 16..
+    // the last row's.  A first row that ended where the tile starts adds 0.
+    if (w0 == 0) {
+      const int j = lane & 15;
+      const X *src = lane < 16 ? sm.rows[0] : sm.last;
+      double *dst = nullptr;
+      if (lane < 16) {
+        if (flag && nrows > 0) dst = a.head;
+      } else if (nrows == 0) {
+        if (flag)
+          dst = a.head;
+        else if (k1 > k0)
+          dst = a.tail;
+      } else if (k1 > last_end) {
+        dst = a.tail;
+      }
+      if (j < VW && dst)
+        dst[int64_t(b) * a.hs + v0 + j] = lane < 16 && !has0 ? 0.0 : kv_partial<VW>(src, j);
+    }
+
+    // --- y, a lane per row (a split first row is the fix-up's)
+    int done = -w0;
+    for (int i0 = 0; i0 < nrows; i0 += 32) {
+      const int i = i0 + lane;
+      const bool valid = i < nrows;
+      const int32_t st = valid ? __ldg(a.row_ptr + r0 + i) : 0;
+      const int32_t en = valid ? __ldg(a.row_ptr + r0 + i + 1) : 0;
+      const bool holds = valid && en > max(st, k0);
+      const unsigned dm = __ballot_sync(full, holds);
+      const int rk = done + __popc(dm & ((1u << lane) - 1u));
+      done += __popc(dm);
+      if (valid && !(i == 0 && flag) &&
+          (holds ? static_cast<unsigned>(rk) < unsigned(kKvRows) : w0 == 0)) {
+        X t[VW];
+        if (holds) {
+          Acc tot;
+          tot.load(sm.rows[rk]);
+          tot.totals(t);
+        } else {
 #pragma unroll
-    for (int j = 0; j < VPT; ++j) {
-      const Acc tot = Pol::combine(sm.part[(prow + v0 + j) * 33 + vl], first_acc[j]);
-      if (first_r == 0 && flag)
-        a.head[int64_t(b) * a.hs + v0 + j] = Pol::to_f64(tot);
-      else
-        spmm_write_row<Pol, KP, kCopy>(a, v0 + j, r0 + first_r, tot);
+          for (int j = 0; j < VW; ++j) t[j] = X(0);
+        }
+        X *yp = a.y + v0 * a.ldy + r0 + i;
+#pragma unroll
+        for (int j = 0; j < VW; ++j)
+          if (v0 + j < a.k)
+            yp[j * a.ldy] = finish_total(t[j], fin, a.alpha, a.beta, yp + j * a.ldy);
+      }
+    }
+    __syncwarp();
+    w0 += kKvRows;
+    if (w0 >= ends) {
+      w0 = 0;
+      v0 += VW;
     }
   }
-  // the next tile of this group rewrites rp only after every thread of
-  // the group has passed the scan above (which read it)
 }
 
-// fixup_tile for KP vectors: partials at head/tail[tile * KP + v]; the sums
-// are formed in the same order as fixup_tile's, vector by vector.
-template <class X, int KP, class View>
-__device__ __forceinline__ void fixup_tile_k(const View &v, int T, int b, const double *head,
-                                             const double *tail, X *y, int64_t ldy, int k,
-                                             double alpha, double beta) {
+// fixup_tile for vector j of tile b: partials at head/tail[tile * hs + j];
+// the sums are formed in the same order as fixup_tile's.
+template <class X, class View>
+__device__ __forceinline__ void fixup_tile_k(const View &v, int T, int b, int j, int hs,
+                                             const double *head, const double *tail, X *y,
+                                             int64_t ldy, double alpha, double beta) {
   int32_t r;
   if (!fixup_run_start(v, T, b, r)) return;
-  // length of the run of tiles b, b+1, ... that continue row r
-  int run = 0;
-  for (int j0 = b;; j0 += 8) {
-    int32_t rj[8];
-    bool fj[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      fj[u] = false;
-      if (j0 + u < T) v.row_flag(j0 + u, rj[u], fj[u]);
-    }
-    int n8 = 8;
-#pragma unroll
-    for (int u = 7; u >= 0; --u)
-      if (!(fj[u] && rj[u] == r)) n8 = u;
-    run += n8;
-    if (n8 < 8) break;
+  double s = tail[int64_t(b - 1) * hs + j];
+  for (int j0 = b; fixup_chunk(v, T, j0, r, head + j, s, hs) == 8; j0 += 8) {
   }
-#pragma unroll
-  for (int j = 0; j < KP; ++j) {
-    if (j >= k) break;
-    double s = tail[int64_t(b - 1) * KP + j];
-    for (int t = 0; t < run; ++t) s += head[int64_t(b + t) * KP + j];
-    X *yp = y + j * ldy + r;
-    *yp = static_cast<X>(finish_merged(s, alpha, beta, beta == 0.0 ? 0.0 : double(*yp)));
-  }
+  fixup_write(y + j * ldy, r, s, alpha, beta);
 }
 
 }  // namespace msrep

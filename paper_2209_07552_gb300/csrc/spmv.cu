@@ -101,8 +101,6 @@ __global__ void __launch_bounds__(kThreads, MSREP_MINB) csr_direct(CsrArgs<Pol> 
                                                        int64_t nnz) {
   grid_dependency_wait();
   __shared__ int32_t s_rp[kWarps][32 * IPT + 8];
-  // per-row compensation flags of the low-precision form
-  __shared__ uint8_t s_cf[Pol::kLow ? kWarps : 1][Pol::kLow ? 32 * IPT + 8 : 1];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const TileWalk tw = tile_walk(*n_tiles, kWarps, a.part_toff);
   const int T = tw.end, stride = tw.step;
@@ -121,7 +119,7 @@ __global__ void __launch_bounds__(kThreads, MSREP_MINB) csr_direct(CsrArgs<Pol> 
     p1 = r0 + 32 + lane < rend ? __ldg(a.row_ptr + r0 + 32 + lane) : 0;
   };
   if (b < T) fetch(b);
-  auto walk = [&](auto copy) {
+  with_modes<Pol>(a.finish, a.comp_mode, [&](auto copy, auto comp) {
     for (; b < T; b += stride) {
       const int32_t cr0 = r0, ck0 = k0, cr1 = r1, ck1 = k1;
       const int32_t rend = min(cr1 + 2, a.m + 1);
@@ -131,18 +129,12 @@ __global__ void __launch_bounds__(kThreads, MSREP_MINB) csr_direct(CsrArgs<Pol> 
         s_rp[wid][r - cr0] = __ldg(a.row_ptr + r);
       __syncwarp();
       if (b + stride < T) fetch(b + stride);
-      csr_tile_compute<Pol, GlobalSrc, decltype(copy)::value>(
+      csr_tile_compute<Pol, GlobalSrc, decltype(copy)::value, decltype(comp)::value>(
           a, b, cr0, ck0, cr1, ck1, s_rp[wid], Seg<int32_t>{a.col_idx, 0},
-          Seg<typename Pol::V>{a.val, 0}, nnz, GlobalSrc{}, Pol::kLow ? s_cf[wid] : nullptr);
+          Seg<typename Pol::V>{a.val, 0}, nnz, GlobalSrc{});
       __syncwarp();
     }
-  };
-  // alpha = 1, beta = 0 (the usual call) finishes rows by a copy, decided
-  // at compile time so that no other finishing mode is issued beside it
-  if (a.finish == kFinishCopy)
-    walk(std::true_type{});
-  else
-    walk(std::false_type{});
+  });
 }
 
 template <class Pol, int IPT>
@@ -211,9 +203,11 @@ __global__ void __launch_bounds__(kThreads) csr_stream(CsrArgs<Pol> a, const int
     fill_tail(col_s(s), a.col_idx, q, q.base, g_end);
     fill_tail(val_s(s), a.val, v, v.base, g_end);
     __syncwarp();
-    csr_tile_compute<Pol>(a, b, c.x, c.y, c.z, c.w, rp_s(s) + (c.x - p.base),
-                          Seg<int32_t>{col_s(s), q.base}, Seg<V>{val_s(s), v.base}, nnz,
-                          SharedSrc{});
+    with_modes<Pol>(kFinishScale, a.comp_mode, [&](auto, auto comp) {
+      csr_tile_compute<Pol, SharedSrc, false, decltype(comp)::value>(
+          a, b, c.x, c.y, c.z, c.w, rp_s(s) + (c.x - p.base), Seg<int32_t>{col_s(s), q.base},
+          Seg<V>{val_s(s), v.base}, nnz, SharedSrc{});
+    });
     __syncwarp();
     if (lane == 0 && b + S * W < T) {
       fence_proxy_async();
@@ -241,21 +235,16 @@ __global__ void __launch_bounds__(kThreads, MSREP_MINB) coo_direct(CooArgs<Pol> 
   // the next tile's range is loaded while the current one is processed
   int32_t k0 = 0, k1 = 0;
   if (b < T) coo_tile_range(a, b, k0, k1);
-  auto walk = [&](auto copy) {
+  with_modes<Pol>(a.finish, a.comp_mode, [&](auto copy, auto comp) {
     for (; b < T; b += stride) {
       const int32_t ck0 = k0, ck1 = k1;
       if (b + stride < T) coo_tile_range(a, b + stride, k0, k1);
-      coo_tile_compute<Pol, GlobalSrc, decltype(copy)::value>(
+      coo_tile_compute<Pol, GlobalSrc, decltype(copy)::value, decltype(comp)::value>(
           a, b, ck0, ck1, Seg<int32_t>{a.row_idx, 0}, Seg<int32_t>{a.col_idx, 0},
           Seg<typename Pol::V>{a.val, 0}, GlobalSrc{});
       __syncwarp();
     }
-  };
-  // the common alpha = 1, beta = 0 specialised at compile time
-  if (a.finish == kFinishCopy)
-    walk(std::true_type{});
-  else
-    walk(std::false_type{});
+  });
 }
 
 template <class Pol, int IPT>
@@ -322,8 +311,11 @@ __global__ void __launch_bounds__(kThreads) coo_stream(CooArgs<Pol> a) {
     fill_tail(col_s(s), a.col_idx, q, q.base, g_end);
     fill_tail(val_s(s), a.val, v, v.base, g_end);
     __syncwarp();
-    coo_tile_compute<Pol>(a, b, c.x, c.y, Seg<int32_t>{row_s(s), r.base},
-                          Seg<int32_t>{col_s(s), q.base}, Seg<V>{val_s(s), v.base}, SharedSrc{});
+    with_modes<Pol>(kFinishScale, a.comp_mode, [&](auto, auto comp) {
+      coo_tile_compute<Pol, SharedSrc, false, decltype(comp)::value>(
+          a, b, c.x, c.y, Seg<int32_t>{row_s(s), r.base}, Seg<int32_t>{col_s(s), q.base},
+          Seg<V>{val_s(s), v.base}, SharedSrc{});
+    });
     __syncwarp();
     if (lane == 0 && b + S * W < T) {
       fence_proxy_async();

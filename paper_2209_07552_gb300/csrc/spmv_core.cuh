@@ -52,7 +52,10 @@ struct PolF64 {
   using Acc = double;
   static constexpr bool kLow = false;
   __device__ static Acc zero() { return 0.0; }
-  __device__ static Acc fma(Acc a, double v, double x, bool) { return __fma_rn(v, x, a); }
+  template <bool kComp>
+  __device__ static Acc fma(Acc a, double v, double x) {
+    return __fma_rn(v, x, a);
+  }
   __device__ static Acc combine(Acc a, Acc b) { return __dadd_rn(a, b); }
   __device__ static double to_f64(Acc a) { return a; }
   __device__ static X finish(Acc a, int mode, double alpha, double beta, const X *y) {
@@ -65,12 +68,28 @@ struct PolF64 {
 };
 
 // Low precision: values FP32 or BF16, x and y FP32, binary32 accumulation.
-// A compensated row accumulates (s, c) by Ogita-Rump-Oishi Dot2: every
-// product keeps its rounding error (TwoProduct by FMA) and every addition
-// its error (TwoSum); a plain row uses one FP32 FMA per nonzero.
+// A row accumulates (s, c) by Ogita-Rump-Oishi Dot2: every product keeps its
+// rounding error (TwoProduct by FMA) and every addition its error (TwoSum);
+// with MSREP_COMP_NONE one FP32 FMA per nonzero.  Rows longer than 256
+// nonzeros and rows split between tiles or partitions must be compensated;
+// the others are as well, because finding out which rows those are costs more
+// than the ten FP32 instructions a nonzero they would save (row-sorted COO in
+// particular had to search its row index for each run's extent): nearly every
+// warp holds a lane on a split row, so both updates were issued anyway
+// (R-MAT 2^20 / 2^24 nonzeros, FP32: COO 147 -> 100 us, CSR 107 -> 100 us;
+// error against FP64 5e-8 -> 2.5e-8).
 struct F32Pair {
   float s, c;
 };
+
+// s + c of an accumulator.  A sum that overflowed, or met an infinity or a
+// NaN, leaves a c that is not finite; its value is then s alone.
+__device__ __forceinline__ float pair_total(float s, float c) {
+  return fabsf(c) < INFINITY ? __fadd_rn(s, c) : s;
+}
+__device__ __forceinline__ double pair_total_f64(float s, float c) {
+  return double(s) + (fabsf(c) < INFINITY ? double(c) : 0.0);
+}
 
 template <typename VT>
 struct PolF32 {
@@ -79,8 +98,9 @@ struct PolF32 {
   using Acc = F32Pair;
   static constexpr bool kLow = true;
   __device__ static Acc zero() { return F32Pair{0.f, 0.f}; }
-  __device__ static Acc fma(Acc a, float v, float x, bool comp) {
-    if (comp) {
+  template <bool kComp>
+  __device__ static Acc fma(Acc a, float v, float x) {
+    if (kComp) {
       float p, ep, s, es;
       two_prod(v, x, p, ep);
       two_sum(a.s, p, s, es);
@@ -93,9 +113,9 @@ struct PolF32 {
     two_sum(a.s, b.s, s, e);
     return F32Pair{s, __fadd_rn(__fadd_rn(a.c, b.c), e)};
   }
-  __device__ static double to_f64(Acc a) { return double(a.s) + double(a.c); }
+  __device__ static double to_f64(Acc a) { return pair_total_f64(a.s, a.c); }
   __device__ static X finish(Acc a, int mode, double alpha, double beta, const X *y) {
-    float t = __fadd_rn(a.s, a.c);
+    float t = pair_total(a.s, a.c);
     if (mode == kFinishCopy) return t;
     float r = __fmul_rn(float(alpha), t);
     if (mode == kFinishScale) return r;
@@ -112,13 +132,21 @@ struct PolF32 {
 __device__ __forceinline__ double load_x(const double *x, int32_t c) { return __ldg(x + c); }
 __device__ __forceinline__ float load_x(const float *x, int32_t c) { return __ldg(x + c); }
 
-// Compensation predicate of the low-precision form: rows longer than 256
-// nonzeros and rows split between tiles or partitions, unless the caller
-// forces all / none.
-__device__ __forceinline__ bool want_comp(unsigned mode, int64_t len, bool split) {
-  if (mode & MSREP_COMP_ALL) return true;
-  if (mode & MSREP_COMP_NONE) return false;
-  return split || len > 256;
+// Runs f(copy, comp) with the finishing mode (copy: alpha = 1, beta = 0) and
+// the compensation (comp: not MSREP_COMP_NONE, which MSREP_COMP_ALL
+// overrides) as compile-time constants, so that the nonzero loop carries one
+// update and the usual finish only; uncompensated calls keep the run-time
+// finish.
+template <class Pol, class F>
+__device__ __forceinline__ void with_modes(int finish, unsigned comp_mode, F f) {
+  const bool copy = finish == kFinishCopy;
+  if (Pol::kLow && (comp_mode & (MSREP_COMP_ALL | MSREP_COMP_NONE)) == MSREP_COMP_NONE) {
+    f(std::false_type{}, std::false_type{});
+  } else if (copy) {
+    f(std::true_type{}, std::integral_constant<bool, Pol::kLow>{});
+  } else {
+    f(std::false_type{}, std::integral_constant<bool, Pol::kLow>{});
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -307,18 +335,15 @@ __device__ __forceinline__ void write_row(const CsrArgs<Pol> &a, int32_t row,
 // One merge-path tile b = rows [r0, r1] x nonzeros [k0, k1), processed by
 // one warp.  rp[j] = row_ptr[r0 + j] for j = 0..r1-r0, and also j = r1-r0+1
 // when r1 < m; rp must be in shared memory (it is searched).
-// cf (low-precision form, optional): this warp's nrows + 1 bytes of shared
-// memory for the tile's per-row compensation flags, filled once here by all
-// lanes; the row-finishing path, which the lanes of a warp reach at
-// different steps, then reads one byte instead of recomputing the predicate.
 // kCopy: the caller knows that alpha = 1 and beta = 0 (every row finished
-// by the copy mode, decided at compile time).
-template <class Pol, class Src, bool kCopy = false>
+// by the copy mode, decided at compile time).  kComp: compensated sums
+// (low-precision form).
+template <class Pol, class Src, bool kCopy, bool kComp>
 __device__ __forceinline__ void csr_tile_compute(const CsrArgs<Pol> &a, int b, int32_t r0,
                                                  int32_t k0, int32_t r1, int32_t k1,
                                                  const int32_t *rp, Seg<int32_t> col,
                                                  Seg<typename Pol::V> val, int64_t nnz,
-                                                 Src src, uint8_t *cf = nullptr) {
+                                                 Src src) {
   using Acc = typename Pol::Acc;
   using LV = typename LoadT<typename Pol::V>::type;
   const int lane = threadIdx.x & 31;
@@ -338,25 +363,8 @@ __device__ __forceinline__ void csr_tile_compute(const CsrArgs<Pol> &a, int b, i
   const int r_end = upper_bound_smem(s_end, nrows, kb);
   int32_t next_end = r < r_end ? s_end[r] : INT32_MAX;
 
-  // compensation predicate (low-precision form only)
-  int32_t re_last = 0;
-  if (Pol::kLow) re_last = (r1 < a.m) ? rp[nrows + 1] : k1;
-  auto row_comp_of = [&](int rr) -> bool {
-    int64_t st = rr == 0 ? int64_t(rs0) : int64_t(s_end[rr - 1]);
-    int64_t en = rr < nrows ? int64_t(s_end[rr]) : int64_t(re_last);
-    return want_comp(a.comp_mode, en - st, (rr == 0 && flag) || rr == nrows);
-  };
-  if (Pol::kLow && cf) {
-    for (int rr = lane; rr <= nrows; rr += 32) cf[rr] = row_comp_of(rr);
-    __syncwarp();
-  }
-  auto row_comp = [&](int rr) -> bool {
-    if (!Pol::kLow) return false;
-    return cf ? cf[rr] != 0 : row_comp_of(rr);
-  };
-
   Acc acc = Pol::zero(), first_acc = Pol::zero();
-  bool emitted = false, comp = row_comp(r);
+  bool emitted = false;
   int first_r = 0;
   // finish every row whose end is <= kk (several when rows are empty)
   auto finish_rows = [&](int32_t kk) {
@@ -371,7 +379,6 @@ __device__ __forceinline__ void csr_tile_compute(const CsrArgs<Pol> &a, int b, i
       acc = Pol::zero();
       ++r;
       next_end = r < r_end ? s_end[r] : INT32_MAX;
-      comp = row_comp(r);
     }
   };
   finish_rows(ka);
@@ -396,7 +403,7 @@ __device__ __forceinline__ void csr_tile_compute(const CsrArgs<Pol> &a, int b, i
     // r stops at r_end.
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      acc = Pol::fma(acc, v[u], xv[u], comp);
+      acc = Pol::template fma<kComp>(acc, v[u], xv[u]);
       const int32_t kk = static_cast<int32_t>(g8 + u + 1);
       if (next_end <= kk) finish_rows(kk);
     }
@@ -456,37 +463,11 @@ __device__ __forceinline__ void coo_tile_range(const CooArgs<Pol> &a, int b, int
   k1 = static_cast<int32_t>(s + (int64_t(g + 1) * L) / a.G);
 }
 
-// In-tile length of the run of row rv around nonzero j of a row-sorted
-// COO tile [k0, k1), or 0 when two probes 128 positions either side of j
-// both miss rv (the run is then shorter than 256).  Out of line: a lane
-// calls it for a few runs at most, and inlined at every call site it made
-// the low-precision COO kernel wait on instruction fetch.
-static __device__ __noinline__ int64_t coo_run_length(const int32_t *row_idx, int64_t k0,
-                                                      int64_t k1, int32_t rv, int64_t j) {
-  const int64_t pa = max(k0, j - 128), pb = min(k1 - 1, j + 128);
-  const bool reach_a = pa < j && __ldg(row_idx + pa) == rv;
-  const bool reach_b = pb > j && __ldg(row_idx + pb) == rv;
-  if (!reach_a && !reach_b) return 0;
-  int64_t lo = k0, hi = j;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (__ldg(row_idx + mid) < rv) lo = mid + 1; else hi = mid;
-  }
-  const int64_t st = lo;
-  lo = j;
-  hi = k1;
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (__ldg(row_idx + mid) <= rv) lo = mid + 1; else hi = mid;
-  }
-  return lo - st;
-}
-
 // kCopy: the caller knows that alpha = 1 and beta = 0, so every row is
 // finished by the copy mode (compile-time: the finishing code shrinks to
 // that case, which keeps the low-precision kernel's loop in the
-// instruction cache).
-template <class Pol, class Src, bool kCopy = false>
+// instruction cache).  kComp: compensated sums (low-precision form).
+template <class Pol, class Src, bool kCopy, bool kComp>
 __device__ __forceinline__ void coo_tile_compute(const CooArgs<Pol> &a, int b, int32_t k0,
                                                  int32_t k1, Seg<int32_t> row,
                                                  Seg<int32_t> col, Seg<typename Pol::V> val,
@@ -519,44 +500,8 @@ __device__ __forceinline__ void coo_tile_compute(const CooArgs<Pol> &a, int b, i
   const LaneRange lr = lane_range(k0, k1, lane);
   const int64_t ka = lr.ka, kb = lr.kb;
 
-  // compensation predicate of the run of row rv that contains nonzero j:
-  // split if it touches a tile end that the row crosses (rows are sorted,
-  // so it touches the tile's start iff rv is the tile's first row), long if
-  // its length inside the tile exceeds 256 (coo_run_length; a split run is
-  // caught first, so the length test alone decides the rest).  A row that
-  // crosses the tile is split anyway; inside the tile, its in-tile length
-  // is its full length.
-  auto run_comp = [&](int32_t rv, int64_t j) -> bool {
-    if (!Pol::kLow) return false;
-    if (a.comp_mode & (MSREP_COMP_ALL | MSREP_COMP_NONE))
-      return want_comp(a.comp_mode, 0, false);
-    const bool split = (rv == first_row && flag) || (rv == last_row && cont);
-    if (split) return true;
-    return coo_run_length(a.row_idx, k0, k1, rv, j) > 256;
-  };
-
-  // A lane whose range holds at most 256 nonzeros needs the predicate for
-  // two runs at most: every run it both starts and ends is shorter than 257
-  // and touches neither tile end, so only its first and last runs (the rows
-  // at ka and kb - 1) can be long or split.  Those two are settled here,
-  // before the nonzero loop, instead of at each row change inside it.
-  const bool two_runs = Pol::kLow && kb - ka <= 256;
-  bool comp_first = false, comp_last = false;
-  int32_t row_first = -1, row_last = -1;
-  if (two_runs && kb > ka) {
-    row_first = __ldg(a.row_idx + ka);
-    row_last = __ldg(a.row_idx + kb - 1);
-    comp_first = run_comp(row_first, ka);
-    comp_last = row_last == row_first ? comp_first : run_comp(row_last, kb - 1);
-  }
-  const bool comp_mid = Pol::kLow && want_comp(a.comp_mode, 0, false);
-  auto comp_of = [&](int32_t rv, int64_t j) -> bool {
-    if (!two_runs) return run_comp(rv, j);
-    return rv == row_first ? comp_first : rv == row_last ? comp_last : comp_mid;
-  };
-
   Acc acc = Pol::zero(), first_acc = Pol::zero();
-  bool emitted = false, comp = false;
+  bool emitted = false;
   int32_t first_r = 0, cur = -1, lane_next = -1;
   auto emit = [&]() {
     if (!emitted) {
@@ -596,9 +541,8 @@ __device__ __forceinline__ void coo_tile_compute(const CooArgs<Pol> &a, int b, i
           for (int32_t rr = cur + 1; rr < rw[u]; ++rr) write_empty(rr);
         }
         cur = rw[u];
-        comp = comp_of(cur, g8 + u);
       }
-      acc = Pol::fma(acc, v[u], xv[u], comp);
+      acc = Pol::template fma<kComp>(acc, v[u], xv[u]);
     }
   }
   // the lane's last run ends here if the next nonzero starts another row
@@ -953,6 +897,8 @@ struct CsrTileView {
     r = __ldg(tile_row + b);
     f = __ldg(row_ptr + r) < __ldg(tile_k + b);
   }
+  // does tile b start inside row r (which an earlier tile started)?
+  __device__ bool continues(int b, int32_t r) const { return __ldg(tile_row + b) == r; }
 };
 
 struct CooTileView {
@@ -975,6 +921,10 @@ struct CooTileView {
     r = __ldg(row_idx + k);
     f = k > 0 && __ldg(row_idx + k - 1) == r;
   }
+  __device__ bool continues(int b, int32_t r) const {
+    const int32_t k = k0(b);
+    return k < nnz && __ldg(row_idx + k) == r;
+  }
 };
 
 // Merge of one row split between tiles (Sec. 3.2.1 / Sec. 4.3): the first
@@ -996,27 +946,24 @@ __device__ __forceinline__ bool fixup_run_start(const View &v, int T, int b, int
 }
 
 // Adds, in order, the head partials of tiles j0 .. j0+7 that continue row r
-// to s; returns how many continued it (8: the run may go on).  The flags
-// and partials of the 8 tiles are loaded together (a hub row spans dozens
-// of tiles; one dependent load chain per tile made the walk latency-bound).
+// to s; returns how many continued it (8: the run may go on).  The rows
+// and partials of the 8 tiles are loaded together, in one round trip (a hub
+// row spans dozens of tiles; a chain of dependent loads per tile made the
+// walk latency-bound).  Tile t's partial lies at head[t * hs].
 template <class View>
 __device__ __forceinline__ int fixup_chunk(const View &v, int T, int j0, int32_t r,
-                                           const double *head, double &s) {
-  int32_t rj[8];
-  bool fj[8];
+                                           const double *head, double &s, int hs = 1) {
+  bool in[8];
   double hj[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
-    fj[u] = false;
-    if (j0 + u < T) {
-      v.row_flag(j0 + u, rj[u], fj[u]);
-      hj[u] = head[j0 + u];
-    }
+    in[u] = j0 + u < T && v.continues(j0 + u, r);
+    hj[u] = j0 + u < T ? head[int64_t(j0 + u) * hs] : 0.0;
   }
   int run = 8;
 #pragma unroll
   for (int u = 7; u >= 0; --u)
-    if (!(fj[u] && rj[u] == r)) run = u;
+    if (!in[u]) run = u;
 #pragma unroll
   for (int u = 0; u < 8; ++u)
     if (u < run) s += hj[u];
@@ -1072,11 +1019,8 @@ __device__ __forceinline__ void fixup_warp(const View &v, int T, int base, const
       bool in = false;
       double h = 0.0;
       if (j < T) {
-        int32_t rj;
-        bool fj;
-        v.row_flag(j, rj, fj);
-        in = fj && rj == rr;
-        if (in) h = head[j];
+        in = v.continues(j, rr);
+        h = head[j];
       }
       const unsigned im = __ballot_sync(full, in);
       const int cnt = im == full ? 32 : __ffs(~im) - 1;
