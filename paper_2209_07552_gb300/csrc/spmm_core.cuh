@@ -350,20 +350,6 @@ struct KvAcc<PolF32<VT>, 1> {
   }
 };
 
-// y of a finished row from its total t (s + c of the low-precision form),
-// rounded as Pol::finish rounds it
-__device__ __forceinline__ double finish_total(double t, int mode, double alpha, double beta,
-                                               const double *y) {
-  return PolF64::finish(t, mode, alpha, beta, y);
-}
-__device__ __forceinline__ float finish_total(float t, int mode, double alpha, double beta,
-                                              const float *y) {
-  if (mode == kFinishCopy) return t;
-  const float r = __fmul_rn(float(alpha), t);
-  if (mode == kFinishScale) return r;
-  return __fmaf_rn(float(beta), *y, r);
-}
-
 // Four consecutive elements at h4 (a multiple of 4): one vector load, or
 // element-wise at the array's end.
 __device__ __forceinline__ void ld4(const int32_t *p, int32_t (&r)[4]) {

@@ -64,13 +64,19 @@ int *kernel_err_ptr() {
 // ---------------------------------------------------------------------------
 
 // Minimum resident blocks per SM asked of the register allocator for the
-// CSR and COO direct-load kernels: 3 (85 registers a thread, 24 warps per
-// SM) was measured fastest at the default tile of 512 on GB300 (R-MAT and
-// Laplacian CSR 108 / 99 us, COO 120 / 114 us; 1 block cap: 121 / 122 and
-// 125 / 134 us; 4: 112 / 95 and 127 / 121 us).
+// COO direct-load kernel: 3 (80 registers a thread, 24 warps per SM) was
+// measured fastest at the default tile of 512 on GB300 (R-MAT and Laplacian
+// 120 / 114 us; 1 block cap: 125 / 134 us; 4: 127 / 121 us).
 #ifndef MSREP_MINB
 #define MSREP_MINB 3
 #endif
+// The same for the CSR kernel: FP64 needs 80 registers (R-MAT / Laplacian 91 /
+// 87 us with 3 blocks, 97 / 90 with 4, which spills); the low-precision forms
+// fit 64 (FP32 71 / 66 us with 4 blocks, 73 / 73 with 3).
+template <class Pol>
+constexpr int csr_blocks() {
+  return Pol::kLow ? 4 : 3;
+}
 constexpr int kWarps = 8;  // warps per block; each warp owns whole tiles
 constexpr int kThreads = 32 * kWarps;
 
@@ -97,49 +103,46 @@ __device__ __forceinline__ void fill_tail(T *dst, const T *arr, const SegCopy &c
 }
 
 template <class Pol, int IPT>
-__global__ void __launch_bounds__(kThreads, MSREP_MINB) csr_direct(CsrArgs<Pol> a, const int32_t *n_tiles,
-                                                       int64_t nnz) {
+__global__ void __launch_bounds__(kThreads, csr_blocks<Pol>()) csr_direct(CsrArgs<Pol> a,
+                                                                          const int32_t *n_tiles,
+                                                                          int32_t nnz) {
   grid_dependency_wait();
-  __shared__ int32_t s_rp[kWarps][32 * IPT + 8];
+  constexpr int kBytes = CsrTileSmem<Pol>::bytes(32 * IPT);
+  __shared__ __align__(16) char s_tile[kWarps * kBytes];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const CsrTileSmem<Pol> sm(s_tile + wid * kBytes, 32 * IPT);
   const TileWalk tw = tile_walk(*n_tiles, kWarps, a.part_toff);
   const int T = tw.end, stride = tw.step;
-  // The next tile's coordinates and its first 64 row pointers are loaded
+  // The next tile's coordinates and its first 96 row pointers are loaded
   // while the current tile is processed, so a tile does not start with two
   // dependent global round trips (coordinates, then row pointers).
   int b = tw.first;
-  int32_t r0 = 0, k0 = 0, r1 = 0, k1 = 0, p0 = 0, p1 = 0;
+  int32_t r0 = 0, k0 = 0, r1 = 0, k1 = 0, p0 = 0, p1 = 0, p2 = 0;
   auto fetch = [&](int t) {
     r0 = __ldg(a.tile_row + t);
     k0 = __ldg(a.tile_k + t);
     r1 = __ldg(a.tile_row + t + 1);
     k1 = __ldg(a.tile_k + t + 1);
-    const int32_t rend = min(r1 + 2, a.m + 1);
-    p0 = r0 + lane < rend ? __ldg(a.row_ptr + r0 + lane) : 0;
-    p1 = r0 + 32 + lane < rend ? __ldg(a.row_ptr + r0 + 32 + lane) : 0;
+    const int32_t *rp = a.row_ptr + r0 + lane;
+    const int n = r1 - r0 - lane;
+    p0 = n >= 0 ? __ldg(rp) : 0;
+    p1 = n >= 32 ? __ldg(rp + 32) : 0;
+    p2 = n >= 64 ? __ldg(rp + 64) : 0;
   };
   if (b < T) fetch(b);
   with_modes<Pol>(a.finish, a.comp_mode, [&](auto copy, auto comp) {
     for (; b < T; b += stride) {
-      const int32_t cr0 = r0, ck0 = k0, cr1 = r1, ck1 = k1;
-      const int32_t rend = min(cr1 + 2, a.m + 1);
-      if (cr0 + lane < rend) s_rp[wid][lane] = p0;
-      if (cr0 + 32 + lane < rend) s_rp[wid][32 + lane] = p1;
-      for (int32_t r = cr0 + 64 + lane; r < rend; r += 32)
-        s_rp[wid][r - cr0] = __ldg(a.row_ptr + r);
-      __syncwarp();
+      const int32_t cr0 = r0, ck0 = k0, cr1 = r1, ck1 = k1, cp0 = p0, cp1 = p1, cp2 = p2;
       if (b + stride < T) fetch(b + stride);
-      csr_tile_compute<Pol, GlobalSrc, decltype(copy)::value, decltype(comp)::value>(
-          a, b, cr0, ck0, cr1, ck1, s_rp[wid], Seg<int32_t>{a.col_idx, 0},
-          Seg<typename Pol::V>{a.val, 0}, nnz, GlobalSrc{});
-      __syncwarp();
+      csr_tile<Pol, decltype(copy)::value, decltype(comp)::value>(a, b, cr0, ck0, cr1, ck1, nnz,
+                                                                  sm, cp0, cp1, cp2);
     }
   });
 }
 
 template <class Pol, int IPT>
 __global__ void __launch_bounds__(kThreads) csr_stream(CsrArgs<Pol> a, const int32_t *n_tiles,
-                                                       int64_t nnz) {
+                                                       int32_t nnz) {
   grid_dependency_wait();
   using V = typename Pol::V;
   using G = StageGeom<V, IPT, 2>;
@@ -199,7 +202,7 @@ __global__ void __launch_bounds__(kThreads) csr_stream(CsrArgs<Pol> a, const int
     SegCopy p, q, v;
     plans(c, p, q, v);
     fill_tail(rp_s(s), a.row_ptr, p, c.x, min(int64_t(c.z) + 2, mp1));
-    const int64_t g_end = min((int64_t(c.w) + 7) & ~int64_t(7), nnz);
+    const int64_t g_end = min((int64_t(c.w) + 7) & ~int64_t(7), int64_t(nnz));
     fill_tail(col_s(s), a.col_idx, q, q.base, g_end);
     fill_tail(val_s(s), a.val, v, v.base, g_end);
     __syncwarp();
@@ -835,10 +838,11 @@ static msrep_status run_csr(const msrep_matrix *A, const msrep_partition *p,
   if (!a.err) return fail(MSREP_ERR_CUDA, "cannot resolve the device error word");
   const bool per_part = (flags & MSREP_SCHED_PER_PARTITION) != 0;
   a.part_toff = per_part ? reinterpret_cast<const int32_t *>(plan + L.off_toff) : nullptr;
+  const int32_t nnz = static_cast<int32_t>(A->nnz);
   MSREP_TRY(launch_tiles(csr_stream<Pol, IPT>, csr_direct<Pol, IPT>,
-                         StageGeom<typename Pol::V, IPT, 2>::BLOCK, 0, MSREP_MINB,
+                         StageGeom<typename Pol::V, IPT, 2>::BLOCK, 0, csr_blocks<Pol>(),
                          (flags & MSREP_STREAM_TMA) == 0, L.tmax, per_part ? p->np : 0, st, a,
-                         n_tiles, A->nnz));
+                         n_tiles, nnz));
   CsrTileView v{a.tile_row, a.tile_k, A->ptr, n_tiles};
   int64_t fg = std::min<int64_t>(ceil_div(L.tmax, 256), 4 * sm_count());
   MSREP_TRY(launch_dependent(fixup_split_rows<typename Pol::X, CsrTileView>, fg, 256, st, 0, v,

@@ -75,9 +75,7 @@ struct PolF64 {
 // the others are as well, because finding out which rows those are costs more
 // than the ten FP32 instructions a nonzero they would save (row-sorted COO in
 // particular had to search its row index for each run's extent): nearly every
-// warp holds a lane on a split row, so both updates were issued anyway
-// (R-MAT 2^20 / 2^24 nonzeros, FP32: COO 147 -> 100 us, CSR 107 -> 100 us;
-// error against FP64 5e-8 -> 2.5e-8).
+// warp holds a lane on a split row, so both updates were issued anyway.
 struct F32Pair {
   float s, c;
 };
@@ -332,6 +330,32 @@ __device__ __forceinline__ void write_row(const CsrArgs<Pol> &a, int32_t row,
   a.y[row] = Pol::finish(v, a.finish, a.alpha, a.beta, a.y + row);
 }
 
+// The row pointers of a tile, 32 rows at a time: row i = at() + lane starts
+// at start(), ends at end() (valid for i <= nrows; end() for i < nrows only).
+// The first 96 come from registers the caller loaded ahead (p0, p1, p2).
+struct RowChunks {
+  const int32_t *row_ptr;  // of the tile's first row
+  int nrows, i0;
+  int32_t cur, nxt, nx2;
+  __device__ __forceinline__ RowChunks(const int32_t *rp, int n, int32_t p0, int32_t p1, int32_t p2)
+      : row_ptr(rp), nrows(n), i0(0), cur(p0), nxt(p1), nx2(p2) {}
+  __device__ __forceinline__ bool more() const { return i0 <= nrows; }
+  __device__ __forceinline__ int row() const { return i0 + (threadIdx.x & 31); }
+  __device__ __forceinline__ int32_t start() const { return cur; }
+  __device__ __forceinline__ int32_t end() const {
+    const int32_t dn = __shfl_down_sync(0xffffffffu, cur, 1);
+    const int32_t up = __shfl_sync(0xffffffffu, nxt, 0);
+    return (threadIdx.x & 31) == 31 ? up : dn;
+  }
+  __device__ __forceinline__ void next() {
+    const int i = i0 + 96 + (threadIdx.x & 31);
+    cur = nxt;
+    nxt = nx2;
+    nx2 = i <= nrows ? __ldg(row_ptr + i) : 0;
+    i0 += 32;
+  }
+};
+
 // One merge-path tile b = rows [r0, r1] x nonzeros [k0, k1), processed by
 // one warp.  rp[j] = row_ptr[r0 + j] for j = 0..r1-r0, and also j = r1-r0+1
 // when r1 < m; rp must be in shared memory (it is searched).
@@ -428,6 +452,205 @@ __device__ __forceinline__ void csr_tile_compute(const CsrArgs<Pol> &a, int b, i
       a.tail[b] = Pol::to_f64(last);
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// CSR tile, direct loads
+// ---------------------------------------------------------------------------
+
+// Shared memory of one warp for csr_tile, for tiles of at most `tile` items
+// (such a tile has at most tile / 2 rows that hold a nonzero of it and end in
+// it), laid out from a 16-byte aligned base.
+template <class Pol>
+struct CsrTileSmem {
+  using X = typename Pol::X;
+  X *sum;         // totals of finished rows, in the order of their ends
+  uint8_t *end;   // per element of the tile: 1 if a row ends with it
+  uint32_t *has;  // bit i: row i holds a nonzero and ends in the tile
+  __host__ __device__ static constexpr int bytes(int tile) {
+    return (int(sizeof(X)) * (tile / 2) + tile + 16 + 4 * (tile / 32 + 1) + 15) & ~15;
+  }
+  __device__ __forceinline__ CsrTileSmem(void *base, int tile) {
+    char *p = static_cast<char *>(base);
+    sum = reinterpret_cast<X *>(p);
+    end = reinterpret_cast<uint8_t *>(p + sizeof(X) * (tile / 2));
+    has = reinterpret_cast<uint32_t *>(end + tile + 16);
+  }
+};
+
+// Total that a finished row gives y, before alpha and beta.
+__device__ __forceinline__ double acc_total(double a) { return a; }
+__device__ __forceinline__ float acc_total(F32Pair a) { return pair_total(a.s, a.c); }
+// y from that total, rounded as Pol::finish rounds it
+__device__ __forceinline__ double finish_total(double t, int mode, double alpha, double beta,
+                                               const double *y) {
+  return PolF64::finish(t, mode, alpha, beta, y);
+}
+__device__ __forceinline__ float finish_total(float t, int mode, double alpha, double beta,
+                                              const float *y) {
+  if (mode == kFinishCopy) return t;
+  const float r = __fmul_rn(float(alpha), t);
+  if (mode == kFinishScale) return r;
+  return __fmaf_rn(float(beta), *y, r);
+}
+
+// Aligned groups of 8 nonzeros [lo, hi) of lane `lane` in a tile [k0, k1),
+// counted from the group that holds k0 (lane_range's split).
+__device__ __forceinline__ void lane_groups(int32_t k0, int32_t k1, int lane, int &lo, int &hi) {
+  const int ng = (k1 >> 3) + ((k1 & 7) != 0) - (k0 >> 3);
+  lo = (lane * ng) >> 5;
+  hi = ((lane + 1) * ng) >> 5;
+}
+
+// One merge-path tile b = rows [r0, r1] x nonzeros [k0, k1), processed by
+// one warp.  p0, p1, p2: row_ptr[r0 + lane], [r0 + 32 + lane] and [r0 + 64 +
+// lane] where those rows are <= r1.
+//
+// The lanes split the aligned groups of 8 nonzeros evenly and sum along
+// their runs; rows that a run boundary splits are merged by a warp segmented
+// scan (csr_tile_compute's sums, bit for bit).  Where rows end is worked out
+// first, a lane per row, into a byte per nonzero, so the nonzero loop tests
+// one bit and a row's end costs a predicated store into shared memory; y is
+// written afterwards, a lane per row.  With row ends walked through the row
+// pointers inside the loop, every end (and each empty row after it) took a
+// divergent path with a dependent shared-memory load and a scattered store.
+//
+// What bounds it: for power-law columns the x gathers, one L1 line lookup per
+// nonzero (without them R-MAT FP64 takes 65 us); FP64 arithmetic does not
+// (91 us without it too).  Measured, whole call, before -> after: R-MAT 2^20 /
+// 2^24 nonzeros FP64 / FP32 / BF16 107 / 104 / 102 -> 90 / 72 / 68 us;
+// Laplacian 2048^2 98 / 98 / 100 -> 87 / 66 / 67 us.  Not kept: groups of 4
+// with the next one loaded ahead (half-sector index reads cost DRAM traffic:
+// Laplacian 102 us), whole runs of 16 at once (R-MAT FP64 144 us, spills),
+// gathers one group ahead and L2 prefetches of the next tile (no change).
+template <class Pol, bool kCopy, bool kComp>
+__device__ __forceinline__ void csr_tile(const CsrArgs<Pol> &a, int b, int32_t r0, int32_t k0,
+                                         int32_t r1, int32_t k1, int32_t nnz,
+                                         const CsrTileSmem<Pol> &sm, int32_t p0, int32_t p1,
+                                         int32_t p2) {
+  using Acc = typename Pol::Acc;
+  using X = typename Pol::X;
+  using LV = typename LoadT<typename Pol::V>::type;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int nrows = r1 - r0;
+  RowChunks rc(a.row_ptr + r0, nrows, p0, p1, p2);
+  const int fin = kCopy ? int(kFinishCopy) : a.finish;
+  const int32_t base = k0 & ~7;  // element e of the tile is nonzero base + e
+  const int lo_e = k0 - base, hi_e = k1 - base;
+  int g, ghi;
+  lane_groups(k0, k1, lane, g, ghi);
+  const int glo = g;
+  int32_t c[8];
+  LV v[8];
+  if (g < ghi) {  // the lane's first group, in flight while the rows are worked out
+    load_group(a.col_idx, int64_t(base) + 8 * g, nnz, c);
+    load_group(a.val, int64_t(base) + 8 * g, nnz, v);
+  }
+
+  for (int i = lane; 16 * i < hi_e; i += 32)
+    reinterpret_cast<int4 *>(sm.end)[i] = make_int4(0, 0, 0, 0);
+  __syncwarp();
+  bool flag = false, has0 = false;
+  int32_t last_end = 0;  // row_ptr[r1]
+  for (; rc.more(); rc.next()) {
+    const int i = rc.row();
+    const int32_t st = rc.start(), en = rc.end();
+    const bool done = i < nrows && en > max(st, k0);
+    const unsigned dm = __ballot_sync(full, done);
+    if (rc.i0 == 0) {
+      flag = __shfl_sync(full, st, 0) < k0;
+      has0 = (dm & 1u) != 0;
+    }
+    if (done) sm.end[en - 1 - base] = 1;
+    if (lane == 0) sm.has[rc.i0 >> 5] = dm;
+    if (nrows - rc.i0 < 32) last_end = __shfl_sync(full, st, nrows - rc.i0);
+  }
+  __syncwarp();
+  // place of the lane's first row end among the tile's
+  int rank0;
+  {
+    int cnt = 0;
+    for (int q = g; q < ghi; ++q) {
+      const uint2 f = reinterpret_cast<const uint2 *>(sm.end)[q];
+      cnt += __popc(f.x) + __popc(f.y);
+    }
+    int inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(full, inc, o);
+      if (lane >= o) inc += t;
+    }
+    rank0 = inc - cnt;
+  }
+
+  Acc acc = Pol::zero(), first_acc = Pol::zero();
+  bool emitted = false;
+  X *out = sm.sum + rank0;
+  for (; g < ghi; ++g) {
+    X xv[8];
+    const int e = 8 * g;
+    if (g > glo) {
+      load_group(a.col_idx, int64_t(base) + e, nnz, c);
+      load_group(a.val, int64_t(base) + e, nnz, v);
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const bool in = e + u >= lo_e && e + u < hi_e;
+      xv[u] = in ? load_x(a.x, c[u]) : X(0);
+      if (!in) v[u] = LV(0);
+    }
+    const uint2 f = reinterpret_cast<const uint2 *>(sm.end)[g];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      acc = Pol::template fma<kComp>(acc, v[u], xv[u]);
+      if ((u < 4 ? f.x >> (8 * u) : f.y >> (8 * (u - 4))) & 1u) {  // a row ends here
+        if (emitted)
+          *out = acc_total(acc);
+        else
+          first_acc = acc;
+        emitted = true;
+        ++out;
+        acc = Pol::zero();
+      }
+    }
+  }
+
+  Acc last;
+  const Acc carry = warp_seg_scan<Pol>(emitted, acc, last);
+  if (emitted) {
+    const Acc tot = Pol::combine(carry, first_acc);
+    if (rank0 == 0 && has0 && flag)
+      a.head[b] = Pol::to_f64(tot);
+    else
+      sm.sum[rank0] = acc_total(tot);
+  }
+  if (lane == 31) {
+    if (nrows == 0) {
+      if (flag)
+        a.head[b] = Pol::to_f64(last);
+      else if (k1 > k0)
+        a.tail[b] = Pol::to_f64(last);
+    } else {
+      if (k1 > last_end) a.tail[b] = Pol::to_f64(last);
+      // a first row that ended where the tile starts adds nothing here
+      if (flag && !has0) a.head[b] = 0.0;
+    }
+  }
+  __syncwarp();
+  // y, a lane per row (a split first row is the fix-up's)
+  int before = 0;
+  for (int i0 = 0; i0 < nrows; i0 += 32) {
+    const int i = i0 + lane;
+    const uint32_t hm = sm.has[i0 >> 5];
+    const int rk = before + __popc(hm & ((1u << lane) - 1u));
+    before += __popc(hm);
+    if (i < nrows && (i > 0 || !flag)) {
+      const X t = ((hm >> lane) & 1u) ? sm.sum[rk] : X(0);
+      a.y[r0 + i] = finish_total(t, fin, a.alpha, a.beta, a.y + r0 + i);
+    }
+  }
+  __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
