@@ -16,9 +16,9 @@
 // them take about 55 us on 152 SMs) and, above that, the instructions around
 // it at 16 warps an SM (87M warp instructions on the R-MAT matrix, k = 8;
 // issue slots 46% used, L1 60%).  Measured on R-MAT 2^20 / 2^24 nonzeros,
-// FP32, the whole call: k = 2 / 4 / 8 113 / 136 / 207 us, against 186 / 345 /
+// FP32, the whole call: k = 2 / 4 / 8 108 / 135 / 206 us, against 186 / 345 /
 // 539 us with row ends walked inside the nonzero loop and y written from
-// there (197M warp instructions at k = 8); 2048^2 Laplacian k = 8 302 against
+// there (197M warp instructions at k = 8); 2048^2 Laplacian k = 8 290 against
 // 481 us.  Three things keep the instructions few:
 //  * where the rows of the tile end is worked out once per tile, a lane per
 //    row, into a bit string in shared memory; the nonzero loop tests one bit
@@ -351,14 +351,17 @@ struct KvAcc<PolF32<VT>, 1> {
 };
 
 // Four consecutive elements at h4 (a multiple of 4): one vector load, or
-// element-wise at the array's end.
+// element-wise at the array's end.  Loads of 16 bytes and less go through L1,
+// which serves the other half of their 32-byte sector to the next load
+// (bypassing it read the halves from L2 and DRAM again: Laplacian FP32 k = 8
+// 301 us against 290).
 __device__ __forceinline__ void ld4(const int32_t *p, int32_t (&r)[4]) {
-  asm("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];"
+  asm("ld.global.nc.v4.b32 {%0, %1, %2, %3}, [%4];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
       : "l"(p));
 }
 __device__ __forceinline__ void ld4(const float *p, float (&r)[4]) {
-  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+  asm("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
       : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3])
       : "l"(p));
 }
@@ -369,7 +372,7 @@ __device__ __forceinline__ void ld4(const double *p, double (&r)[4]) {
 }
 __device__ __forceinline__ void ld4(const bf16_t *p, float (&r)[4]) {
   uint32_t w[2];
-  asm("ld.global.nc.L1::no_allocate.v2.b32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p));
+  asm("ld.global.nc.v2.b32 {%0, %1}, [%2];" : "=r"(w[0]), "=r"(w[1]) : "l"(p));
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     r[2 * i] = __uint_as_float(w[i] << 16);
