@@ -64,7 +64,7 @@ struct Request {
   Clock::time_point t_submit;
   bool x_pinned = false, y_pinned = false;  // page-locked: DMA directly
   // page-locked and mapped: the device address of x / y, which the launch's
-  // copy kernels read and write directly (no per-request copy)
+  // kernels read and write directly (no per-request copy)
   const float *x_map = nullptr;
   float *y_map = nullptr;
   bool done = false;
@@ -74,7 +74,11 @@ struct Request {
 
 struct Context {
   cudaStream_t stream = nullptr;
-  cudaEvent_t done_ev = nullptr;  // end of the launch (also polled)
+  cudaEvent_t done_ev = nullptr;  // end of the launch
+  // end of the launch as the completion thread sees it: the launch's last
+  // kernel writes the launch's number here (page-locked, mapped)
+  volatile uint32_t *flag = nullptr;
+  uint32_t number = 0;
   // timing: launch start (before the x copies), kernels start and end
   cudaEvent_t begin_ev = nullptr, k0_ev = nullptr, k1_ev = nullptr;
   float *x_dev = nullptr, *y_dev = nullptr;    // arenas
@@ -92,7 +96,7 @@ struct Context {
   double *head_k = nullptr, *tail_k = nullptr;
   bool busy = false;      // packed by the scheduler (launching or in flight)
   bool pending = false;   // packed, waiting for its issuing thread
-  bool in_flight = false; // its event has been recorded for this launch
+  bool in_flight = false; // issued: its end may be looked for
   std::vector<BatchItem> ritem;  // per request: its matrix
   std::vector<int64_t> rtiles;   // per request: the matrix's tile count
   std::vector<std::shared_ptr<Request>> reqs;  // in this launch
@@ -119,6 +123,7 @@ struct msrep_server {
   int64_t resident = 0;
   bool stop = false, stop_issuers = false;
   std::thread scheduler, completer;
+  std::atomic<uint64_t> issued{0};  // launches put in flight (for the completion thread)
   std::vector<std::thread> issuers;  // one per context
   // statistics
   std::vector<double> lat_us;     // submit -> y in the caller's buffer
@@ -161,6 +166,13 @@ __global__ void serve_copy(const CopyItem *items, int count) {
   }
 }
 
+// The launch's last kernel: everything before it on the stream has ended, so
+// its results are in place when the host sees the number.
+__global__ void serve_signal(volatile uint32_t *flag, uint32_t number) {
+  __threadfence_system();
+  *flag = number;
+}
+
 static msrep_status launch_copies(const CopyItem *items, int count, cudaStream_t st) {
   if (count == 0) return MSREP_OK;
   serve_copy<<<dim3(32, std::min(count, 1024)), 256, 0, st>>>(items, count);
@@ -181,6 +193,7 @@ static void free_context(Context &c) {
   cudaFreeHost(c.x_pin);
   cudaFreeHost(c.y_pin);
   cudaFreeHost(c.dir_pin);
+  cudaFreeHost(const_cast<uint32_t *>(c.flag));
   if (c.done_ev) cudaEventDestroy(c.done_ev);
   if (c.begin_ev) cudaEventDestroy(c.begin_ev);
   if (c.k0_ev) cudaEventDestroy(c.k0_ev);
@@ -191,11 +204,11 @@ static void free_context(Context &c) {
 
 // Per-launch directory, laid out for the launch's R requests (so that one
 // copy of about 250 bytes a request carries it): the SpMV items (one-vector
-// requests) with their tile offsets and x / y pointers, the copy lists
-// (x in, y out), and the k-vector items with tile and unit offsets and
+// requests) with their tile offsets and x / y pointers, the copy list (x in),
+// and the k-vector items with tile and unit offsets and
 // their x / interleaved-x / y pointers.
 struct LaunchDir {
-  size_t items, toff, xs, ys, cin, cout, itk, toffk, uoffk, xin, xtp, ysk, bytes;
+  size_t items, toff, xs, ys, cin, itk, toffk, uoffk, xin, xtp, ysk, bytes;
   explicit LaunchDir(size_t R) {
     size_t o = 0;
     auto take = [&o](size_t b) {
@@ -208,7 +221,6 @@ struct LaunchDir {
     xs = take(sizeof(void *) * R);
     ys = take(sizeof(void *) * R);
     cin = take(sizeof(CopyItem) * R);
-    cout = take(sizeof(CopyItem) * R);
     itk = take(sizeof(BatchItem) * R);
     toffk = take(sizeof(int64_t) * (R + 1));
     uoffk = take(sizeof(int64_t) * (R + 1));
@@ -227,9 +239,11 @@ static size_t dir_size(int32_t max_items) { return LaunchDir(size_t(max_items)).
 // and y are read and written by the launch's kernels directly: x of a
 // one-vector request is copied into the arena by one copy kernel (the
 // SpMV gathers it at random), x of a k-vector request is read by the
-// interleaving kernel itself, and every mapped y is written by one copy
-// kernel at the end.  Other buffers take one DMA copy each (staged through
-// the pinned arenas when pageable).
+// interleaving kernel itself, and a mapped y is written by the SpMV kernels
+// as they finish its rows, once each, so its way over the host link overlaps
+// their work (a copy kernel at the end took 167 us of a 64-request launch).
+// Other buffers take one DMA copy each (staged through the pinned arenas when
+// pageable).
 static msrep_status launch_context(msrep_server *s, Context &c,
                                    const std::vector<BatchItem> &ritem,
                                    const std::vector<int64_t> &rtiles) {
@@ -242,7 +256,6 @@ static msrep_status launch_context(msrep_server *s, Context &c,
   const void **xs = reinterpret_cast<const void **>(dp + L.xs);
   void **ys = reinterpret_cast<void **>(dp + L.ys);
   CopyItem *cin = reinterpret_cast<CopyItem *>(dp + L.cin);
-  CopyItem *cout = reinterpret_cast<CopyItem *>(dp + L.cout);
   BatchItem *itk = reinterpret_cast<BatchItem *>(dp + L.itk);
   int64_t *toffk = reinterpret_cast<int64_t *>(dp + L.toffk);
   int64_t *uoffk = reinterpret_cast<int64_t *>(dp + L.uoffk);
@@ -251,7 +264,7 @@ static msrep_status launch_context(msrep_server *s, Context &c,
   void **ysk = reinterpret_cast<void **>(dp + L.ysk);
 
   int64_t xo = 0, yo = 0, xto = 0, tt = 0, ttk = 0, utk = 0;
-  int n1 = 0, nk = 0, nci = 0, nco = 0;
+  int n1 = 0, nk = 0, nci = 0;
   c.y_off.clear();
   MSREP_CUDA_TRY(cudaEventRecord(c.begin_ev, c.stream));
   for (size_t i = 0; i < R; ++i) {
@@ -271,12 +284,13 @@ static msrep_status launch_context(msrep_server *s, Context &c,
       std::memcpy(c.x_pin + xo, r->x, xb);
       MSREP_CUDA_TRY(cudaMemcpyAsync(c.x_dev + xo, c.x_pin + xo, xb, cudaMemcpyHostToDevice, c.stream));
     }
+    float *ydst = r->y_map ? r->y_map : c.y_dev + yo;  // where they write its y
     if (r->k == 1) {
       it[n1] = bi;
       toff[n1] = tt;
       tt += rtiles[i];
       xs[n1] = xsrc;
-      ys[n1] = c.y_dev + yo;
+      ys[n1] = ydst;
       ++n1;
     } else {
       itk[nk] = bi;
@@ -287,11 +301,10 @@ static msrep_status launch_context(msrep_server *s, Context &c,
       utk += batched_k_units(rtiles[i], r->k);
       xin[nk] = xsrc;
       xtp[nk] = c.xt_dev + xto;
-      ysk[nk] = c.y_dev + yo;
+      ysk[nk] = ydst;
       xto += int64_t(bi.n) * kBatchWidth;
       ++nk;
     }
-    if (r->y_map) cout[nco++] = CopyItem{c.y_dev + yo, r->y_map, int64_t(bi.m) * r->k};
     xo += nx;
     yo += int64_t(bi.m) * r->k;
   }
@@ -317,7 +330,6 @@ static msrep_status launch_context(msrep_server *s, Context &c,
                                reinterpret_cast<void *const *>(dd + L.ysk), c.head_k, c.tail_k, 0,
                                c.stream));
   MSREP_CUDA_TRY(cudaEventRecord(c.k1_ev, c.stream));
-  MSREP_TRY(launch_copies(reinterpret_cast<const CopyItem *>(dd + L.cout), nco, c.stream));
   for (size_t i = 0; i < R; ++i) {
     const auto &r = c.reqs[i];
     if (r->y_map) continue;
@@ -326,6 +338,8 @@ static msrep_status launch_context(msrep_server *s, Context &c,
     MSREP_CUDA_TRY(cudaMemcpyAsync(dst, c.y_dev + c.y_off[i], sizeof(float) * ylen,
                                    cudaMemcpyDeviceToHost, c.stream));
   }
+  serve_signal<<<1, 1, 0, c.stream>>>(c.flag, ++c.number);
+  MSREP_CUDA_TRY(cudaGetLastError());
   MSREP_CUDA_TRY(cudaEventRecord(c.done_ev, c.stream));
   return MSREP_OK;
 }
@@ -422,7 +436,10 @@ static void issuer_loop(msrep_server *s, size_t ci) {
     lk.lock();
     c.pending = false;
     s->host_us.push_back(host);
-    if (st == MSREP_OK) c.in_flight = true;  // only now may its event be polled
+    if (st == MSREP_OK) {
+      c.in_flight = true;  // only now may its end be looked for
+      s->issued.fetch_add(1);
+    }
     s->cv_flight.notify_all();
     if (st != MSREP_OK) {
       // fail the requests of this launch; the context stays usable
@@ -445,47 +462,60 @@ static void issuer_loop(msrep_server *s, size_t ci) {
 }
 
 // Completion thread.  With nothing issued it sleeps on cv_flight; while
-// any launch is in flight it polls the contexts' events back to back
+// any launch is in flight it polls the contexts' flags back to back
 // (yielding between sweeps): a timed sleep between polls would add the
-// kernel's timer slack, tens of microseconds, to every request.
+// kernel's timer slack, tens of microseconds, to every request.  The flags
+// are plain host memory and the list of contexts in flight is only read again
+// when a launch was issued: polling events took the driver's lock, and the
+// list the server's, on every sweep, and the submitting threads waited for
+// both.  A launch whose flag does not come is asked about
+// through its event every kEventPolls sweeps, which is how a failed one shows.
+constexpr int kEventPolls = 4096;
 static void completion_loop(msrep_server *s) {
   cudaSetDevice(s->cfg.device);
+  std::vector<Context *> flying;
+  uint64_t seen = 0;
+  int sweeps = 0;
   for (;;) {
-    {
+    if (flying.empty() || s->issued.load() != seen) {
       std::unique_lock<std::mutex> lk(s->mu);
       bool any = false;
       s->cv_flight.wait(lk, [&] {
-        bool flying = false;
         any = false;
+        flying.clear();
+        seen = s->issued.load();
         for (auto &c : s->ctx) {
           any |= c.busy;
-          flying |= c.busy && c.in_flight;
+          if (c.busy && c.in_flight) flying.push_back(&c);
         }
-        return flying || (s->stop && s->queue.empty() && !any);
+        return !flying.empty() || (s->stop && s->queue.empty() && !any);
       });
-      if (s->stop && s->queue.empty() && !any) return;
+      if (flying.empty()) return;
     }
     bool progressed = false;
-    for (auto &c : s->ctx) {
-      bool flying;
-      {
-        std::lock_guard<std::mutex> lk(s->mu);
-        flying = c.busy && c.in_flight;
+    const bool ask = ++sweeps % kEventPolls == 0;
+    for (size_t f = 0; f < flying.size(); ++f) {
+      Context &c = *flying[f];
+      cudaError_t q = cudaErrorNotReady;
+      if (*c.flag == c.number) {
+        std::atomic_thread_fence(std::memory_order_acquire);
+        q = cudaEventSynchronize(c.done_ev);  // recorded right behind the flag's kernel
+      } else if (ask) {
+        q = cudaEventQuery(c.done_ev);
       }
-      if (!flying) continue;
-      const cudaError_t q = cudaEventQuery(c.done_ev);
       if (q == cudaErrorNotReady) continue;
       progressed = true;
+      flying.erase(flying.begin() + f--);
       // results to the callers' buffers, outside the lock
       for (size_t i = 0; i < c.reqs.size(); ++i) {
         auto &r = c.reqs[i];
+        if (q != cudaSuccess || r->y_pinned) continue;
         int32_t m;
         {
           std::lock_guard<std::mutex> lk(s->mu);
           m = s->mats[r->matrix].m;
         }
-        if (q == cudaSuccess && !r->y_pinned)
-          std::memcpy(r->y, c.y_pin + c.y_off[i], sizeof(float) * size_t(m) * r->k);
+        std::memcpy(r->y, c.y_pin + c.y_off[i], sizeof(float) * size_t(m) * r->k);
       }
       float span_ms = 0.f, kern_ms = 0.f;
       const bool timed = q == cudaSuccess &&
@@ -573,6 +603,7 @@ msrep_status msrep_serve_create(const msrep_serve_config *cfg, msrep_server **ou
                cudaMallocHost(&c.x_pin, cfg->arena_bytes) == cudaSuccess &&
                cudaMallocHost(&c.y_pin, cfg->arena_bytes) == cudaSuccess &&
                cudaMallocHost(&c.dir_pin, c.dir_bytes) == cudaSuccess &&
+               cudaMallocHost(const_cast<uint32_t **>(&c.flag), 64) == cudaSuccess &&
                cudaMalloc(&c.xt_dev, sizeof(float) * c.xt_floats) == cudaSuccess &&
                cudaMalloc(&c.head_k, sizeof(double) * cfg->max_tiles * kBatchWidth) == cudaSuccess &&
                cudaMalloc(&c.tail_k, sizeof(double) * cfg->max_tiles * kBatchWidth) == cudaSuccess &&
@@ -583,6 +614,7 @@ msrep_status msrep_serve_create(const msrep_serve_config *cfg, msrep_server **ou
       return fail(MSREP_ERR_OOM, "cannot allocate the launch contexts");
     }
   }
+  for (auto &c : s->ctx) *c.flag = 0;
   s->resident = per_ctx * cfg->contexts;
   msrep_server *raw = s.release();
   raw->scheduler = std::thread(scheduler_loop, raw);
@@ -740,7 +772,7 @@ msrep_status msrep_serve_submit(msrep_server *s, int64_t id, int32_t k, const fl
     r->y_map = static_cast<float *>(const_cast<void *>(mapped(y, r->y_pinned)));
     cudaGetLastError();
   }
-  std::lock_guard<std::mutex> lk(s->mu);
+  std::unique_lock<std::mutex> lk(s->mu);
   if (s->stop) return fail(MSREP_ERR_SHUTDOWN, "server is stopping");
   auto it = s->mats.find(id);
   if (it == s->mats.end() || it->second.dying)
@@ -755,6 +787,7 @@ msrep_status msrep_serve_submit(msrep_server *s, int64_t id, int32_t k, const fl
   s->reqs[r->id] = r;
   s->queue.push_back(r);
   s->submitted++;
+  lk.unlock();  // the scheduler wakes to a free lock
   s->cv_work.notify_one();
   return ok();
 }
