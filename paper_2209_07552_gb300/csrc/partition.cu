@@ -117,6 +117,9 @@ __device__ __forceinline__ int32_t path_row(const int32_t *__restrict__ ptr,
 // Alg. 2 / Alg. 4: metadata, one thread per partition
 // ---------------------------------------------------------------------------
 
+// Rows a warp search covers in two rounds (part_meta_compressed).
+constexpr int kNearRows = 33 * 32;
+
 // Cut rules of part_meta_compressed.
 enum : int { kCutNonzeros = 0, kCutMergePath = 1, kCutRowBlock = 2 };
 
@@ -140,6 +143,7 @@ __global__ void part_meta_compressed(const int32_t *__restrict__ ptr,
   const bool lead = (threadIdx.x & 31) == 0;
   if (i > np) return;  // warp-uniform
   int64_t s, e;
+  int32_t sr = -1;  // the row that owns s, where the cut found it
   if (cut == kCutRowBlock) {
     const int32_t r0 = static_cast<int32_t>((i * n_major) / np);
     s = __ldg(ptr + r0);
@@ -166,22 +170,21 @@ __global__ void part_meta_compressed(const int32_t *__restrict__ ptr,
     e = d1 - R1 - 1;
   } else {
     s = (i * nnz) / np;
-    if (plan_D) {
-      // level-1 cut of the tile plan: (R(s_i), s_i) with R over [0, n_major]
-      int32_t R;
-      if (i == 0)
-        R = 0;
-      else if (i == np)
-        R = n_major;
-      else
-        R = last_le_warp(ptr, 0, n_major, s);
-      if (lead) {
-        plan_R[i] = R;
-        plan_D[i] = (i == 0) ? 0 : s + R;
-      }
+    // level-1 cut of the tile plan: (R(s_i), s_i) with R over [0, n_major];
+    // between the first and last cuts s_i < nnz (or nnz = 0), where R is also
+    // the row that owns s_i
+    int32_t R = 0;
+    if (i == np)
+      R = n_major;
+    else if (i > 0 || nnz > 0)
+      R = last_le_warp(ptr, 0, n_major, s);
+    if (plan_D && lead) {
+      plan_R[i] = i == 0 ? 0 : R;
+      plan_D[i] = i == 0 ? 0 : s + R;
     }
     if (i == np) return;
     e = ((i + 1) * nnz) / np - 1;
+    sr = R;
   }
   if (e < s) {
     if (lead) {
@@ -193,8 +196,12 @@ __global__ void part_meta_compressed(const int32_t *__restrict__ ptr,
     }
     return;
   }
-  const int32_t sr = last_le_warp(ptr, 0, n_major - 1, s);
-  const int32_t er = last_le_warp(ptr, sr, n_major - 1, e);
+  if (sr < 0) sr = last_le_warp(ptr, 0, n_major - 1, s);
+  // the last row is rarely far from the first: one probe brackets it
+  int32_t hi = n_major - 1;
+  if (hi - sr > kNearRows && static_cast<int64_t>(__ldg(ptr + sr + kNearRows)) > e)
+    hi = sr + kNearRows - 1;
+  const int32_t er = last_le_warp(ptr, sr, hi, e);
   if (lead) {
     start_idx[i] = static_cast<int32_t>(s);
     end_idx[i] = static_cast<int32_t>(e);
@@ -303,21 +310,38 @@ __device__ T block_exclusive_scan(T v, T &total) {
   return base + inc - v;
 }
 
-// local_off[i] = sum_{j<i} (end_major[j] - start_major[j] + 2) (CSR/CSC).
+// The two scans over partitions (CSR/CSC), a block each: local_off[i] =
+// sum_{j<i} (end_major[j] - start_major[j] + 2), and the tile plan's first
+// tiles, tile_off[i] = sum_{j<i} ceil((D[j+1] - D[j]) / tile).  Either array
+// may be null (not wanted); block 0 takes the first one wanted.
 __global__ void __launch_bounds__(1024)
-    local_off_scan(const int32_t *start_major, const int32_t *end_major,
-                   int32_t np, int64_t *local_off) {
+    part_scans(const int32_t *start_major, const int32_t *end_major, int32_t np,
+               int64_t *local_off, const int64_t *D, int32_t tile, int32_t *tile_off) {
   grid_dependency_wait();
+  const bool tiles = tile_off && (blockIdx.x == 1 || !local_off);
   int64_t carry = 0;
   for (int32_t base = 0; base < np; base += blockDim.x) {
-    int32_t i = base + threadIdx.x;
-    int64_t len = (i < np) ? int64_t(end_major[i]) - start_major[i] + 2 : 0;
+    const int32_t i = base + threadIdx.x;
+    int64_t len = 0;
+    if (i < np)
+      len = tiles ? (D[i + 1] - D[i] + tile - 1) / tile
+                  : int64_t(end_major[i]) - start_major[i] + 2;
     int64_t total;
-    int64_t ex = block_exclusive_scan<int64_t>(len, total);
-    if (i < np) local_off[i] = carry + ex;
+    const int64_t ex = block_exclusive_scan<int64_t>(len, total);
+    if (i < np) {
+      if (tiles)
+        tile_off[i] = static_cast<int32_t>(carry + ex);
+      else
+        local_off[i] = carry + ex;
+    }
     carry += total;
   }
-  if (threadIdx.x == 0) local_off[np] = carry;
+  if (threadIdx.x == 0) {
+    if (tiles)
+      tile_off[np] = static_cast<int32_t>(carry);
+    else
+      local_off[np] = carry;
+  }
 }
 
 // Local row_ptr / col_ptr (Alg. 2/4 inner loop, computed on the GPU as in
@@ -328,17 +352,17 @@ __global__ void __launch_bounds__(1024)
 // forward from there, so the work is spread evenly whatever P and the
 // partitions' row spans are.  Entry j of partition i: 0 (j = 0),
 // end - start + 1 (j = span + 1), else ptr[start_major + j] - start_idx.
+// Block `block` of `blocks`.
 template <bool kVec>
-__global__ void __launch_bounds__(256)
+__device__ __forceinline__ void
     local_fill_compressed(const int32_t *__restrict__ ptr, const int32_t *start_idx,
                           const int32_t *end_idx, const int32_t *start_major,
                           const int32_t *end_major, const int64_t *local_off, int32_t np,
-                          int32_t *local) {
-  grid_dependency_wait();
+                          int32_t *local, int block, int blocks) {
   const int64_t total = local_off[np];
   const int lane = threadIdx.x & 31;
-  const int64_t warps = int64_t(gridDim.x) * (blockDim.x >> 5);
-  for (int64_t w0 = (blockIdx.x * int64_t(blockDim.x >> 5) + (threadIdx.x >> 5)) * 256;
+  const int64_t warps = int64_t(blocks) * (blockDim.x >> 5);
+  for (int64_t w0 = (block * int64_t(blockDim.x >> 5) + (threadIdx.x >> 5)) * 256;
        w0 < total; w0 += warps * 256) {
     // partitions of the warp's first and last entries (warp-uniform)
     const int32_t ia = last_le_warp(local_off, 0, np - 1, w0);
@@ -446,42 +470,57 @@ __global__ void __launch_bounds__(256)
 // [D_i, D_{i+1}) is split into ceil(len / tile) equal pieces
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(1024)
-    plan_scan(const int64_t *D, int32_t np, int32_t tile, int32_t *tile_off) {
-  grid_dependency_wait();
-  int64_t carry = 0;
-  for (int32_t base = 0; base < np; base += blockDim.x) {
-    int32_t i = base + threadIdx.x;
-    int64_t g = 0;
-    if (i < np) g = (D[i + 1] - D[i] + tile - 1) / tile;
-    int64_t total;
-    int64_t ex = block_exclusive_scan<int64_t>(g, total);
-    if (i < np) tile_off[i] = static_cast<int32_t>(carry + ex);
-    carry += total;
-  }
-  if (threadIdx.x == 0) tile_off[np] = static_cast<int32_t>(carry);
-}
-
-__global__ void plan_tiles(const int32_t *__restrict__ ptr, int32_t n_major,
-                           int64_t nnz, int32_t np, const int64_t *D,
-                           const int32_t *R, const int32_t *tile_off,
-                           int32_t *tile_row, int32_t *tile_k) {
-  grid_dependency_wait();
-  const int32_t i = blockIdx.x;
-  const int32_t t0 = tile_off[i], G = tile_off[i + 1] - t0;
-  const int64_t d0 = D[i], len = D[i + 1] - d0;
-  const int32_t lo = R[i], hi = R[i + 1];
-  for (int32_t g = threadIdx.x; g < G; g += blockDim.x) {
-    int64_t d = d0 + (static_cast<int64_t>(g) * len) / G;
-    int32_t r = path_row(ptr, lo, hi, d);
-    tile_row[t0 + g] = r;
-    tile_k[t0 + g] = static_cast<int32_t>(d - r);
-  }
-  if (i == np - 1 && threadIdx.x == 0) {
-    const int32_t T = tile_off[np];
+// A thread per tile t: its partition is the last i with tile_off[i] <= t (a
+// partition without tiles shares its offset with the next), its diagonal the
+// g-th even cut of that partition's stretch.  (A block per partition left a
+// matrix in one partition to 128 threads: 462 us for 2^24 nonzeros.)
+__device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32_t n_major,
+                                          int64_t nnz, int32_t np, const int64_t *D,
+                                          const int32_t *R, const int32_t *tile_off,
+                                          int32_t *tile_row, int32_t *tile_k, int64_t t) {
+  const int32_t T = tile_off[np];
+  if (t > T) return;
+  if (t == T) {
     tile_row[T] = n_major;
     tile_k[T] = static_cast<int32_t>(nnz);
+    return;
   }
+  int32_t lo = 0, hi = np - 1;
+  while (lo < hi) {
+    const int32_t mid = lo + (hi - lo + 1) / 2;
+    if (__ldg(tile_off + mid) <= t)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  const int32_t t0 = __ldg(tile_off + lo), G = __ldg(tile_off + lo + 1) - t0;
+  const int64_t d0 = __ldg(D + lo), len = __ldg(D + lo + 1) - d0;
+  const int64_t d = d0 + ((t - t0) * len) / G;
+  const int32_t r = path_row(ptr, __ldg(R + lo), __ldg(R + lo + 1), d);
+  tile_row[t] = r;
+  tile_k[t] = static_cast<int32_t>(d - r);
+}
+
+// What the two scans lead to, in one launch: blocks [0, plan_blocks) write
+// the tile plan, the others the local pointers.  A partitioning is a chain of
+// short dependent launches, so its time is their number times a few
+// microseconds: five took 21.8 us for R-MAT 2^20 / 2^24 nonzeros in 2368
+// partitions with local pointers, three take 15.7.
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+    part_fill(const int32_t *__restrict__ ptr, int32_t n_major, int64_t nnz, int32_t np,
+              const int64_t *D, const int32_t *R, const int32_t *tile_off, int32_t *tile_row,
+              int32_t *tile_k, int plan_blocks, const int32_t *start_idx, const int32_t *end_idx,
+              const int32_t *start_major, const int32_t *end_major, const int64_t *local_off,
+              int32_t *local) {
+  grid_dependency_wait();
+  const int b = static_cast<int>(blockIdx.x);
+  if (b < plan_blocks)
+    plan_tile(ptr, n_major, nnz, np, D, R, tile_off, tile_row, tile_k,
+              b * int64_t(blockDim.x) + threadIdx.x);
+  else
+    local_fill_compressed<kVec>(ptr, start_idx, end_idx, start_major, end_major, local_off, np,
+                                local, b - plan_blocks, static_cast<int>(gridDim.x) - plan_blocks);
 }
 
 // ---------------------------------------------------------------------------
@@ -887,32 +926,31 @@ static msrep_status partition_compressed(const msrep_matrix *A,
       (flags & MSREP_PART_MERGE_PATH) ? int(kCutMergePath)
                                       : (flags & MSREP_PART_ROW_BLOCK) ? int(kCutRowBlock)
                                                                        : int(kCutNonzeros)));
-  if (p->local_off) {
-    MSREP_TRY(launch_dependent(local_off_scan, 1, 1024, st, 0,
+  int32_t *toff = plan ? reinterpret_cast<int32_t *>(plan + L.off_toff) : nullptr;
+  if (toff || p->local_off)
+    MSREP_TRY(launch_dependent(part_scans, toff && p->local_off ? 2 : 1, 1024, st, 0,
                                static_cast<const int32_t *>(p->start_major),
-                               static_cast<const int32_t *>(p->end_major), p->np, p->local_off));
-    if (p->local) {
-      // at most m + 2 np entries (n + 2 np for CSC)
-      const int64_t most = int64_t(n_major) + 2 * int64_t(p->np);
-      const int grid = static_cast<int>(
-          std::max<int64_t>(1, std::min<int64_t>(ceil_div(most, 8 * 256), 8 * sm_count())));
-      if ((reinterpret_cast<uintptr_t>(p->local) & 15) == 0)
-        MSREP_TRY(launch_dependent(local_fill_compressed<true>, grid, 256, st, 0, A->ptr,
-                                   p->start_idx, p->end_idx, p->start_major, p->end_major,
-                                   p->local_off, p->np, p->local));
-      else
-        MSREP_TRY(launch_dependent(local_fill_compressed<false>, grid, 256, st, 0, A->ptr,
-                                   p->start_idx, p->end_idx, p->start_major, p->end_major,
-                                   p->local_off, p->np, p->local));
-    }
-  }
-  if (plan) {
-    int32_t *toff = reinterpret_cast<int32_t *>(plan + L.off_toff);
-    int32_t *trow = reinterpret_cast<int32_t *>(plan + L.off_row);
-    int32_t *tk = reinterpret_cast<int32_t *>(plan + L.off_k);
-    MSREP_TRY(launch_dependent(plan_scan, 1, 1024, st, 0, D, p->np, tile, toff));
-    MSREP_TRY(launch_dependent(plan_tiles, p->np, 128, st, 0, A->ptr, n_major, A->nnz, p->np, D,
-                               R, toff, trow, tk));
+                               static_cast<const int32_t *>(p->end_major), p->np, p->local_off,
+                               static_cast<const int64_t *>(D), tile, toff));
+  if (toff || p->local) {
+    // a thread per tile, the one past the last writes the closing entry
+    const int plan_blocks = toff ? static_cast<int>(ceil_div(L.tmax + 1, 256)) : 0;
+    // at most m + 2 np local entries (n + 2 np for CSC)
+    const int64_t most = int64_t(n_major) + 2 * int64_t(p->np);
+    const int fill_blocks =
+        p->local ? static_cast<int>(std::max<int64_t>(
+                       1, std::min<int64_t>(ceil_div(most, 8 * 256), 8 * sm_count())))
+                 : 0;
+    const auto fill = (reinterpret_cast<uintptr_t>(p->local) & 15) == 0 ? part_fill<true>
+                                                                        : part_fill<false>;
+    int32_t *trow = plan ? reinterpret_cast<int32_t *>(plan + L.off_row) : nullptr;
+    int32_t *tk = plan ? reinterpret_cast<int32_t *>(plan + L.off_k) : nullptr;
+    MSREP_TRY(launch_dependent(fill, plan_blocks + fill_blocks, 256, st, 0, A->ptr, n_major,
+                               A->nnz, p->np, static_cast<const int64_t *>(D),
+                               static_cast<const int32_t *>(R),
+                               static_cast<const int32_t *>(toff), trow, tk, plan_blocks,
+                               p->start_idx, p->end_idx, p->start_major, p->end_major,
+                               p->local_off, p->local));
   }
   if (side) MSREP_TRY(join_side(st, side));
   return ok();
