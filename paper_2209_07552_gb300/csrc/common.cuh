@@ -206,25 +206,42 @@ __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// Launches a kernel that depends on the previous one on the stream as a
-// programmatic dependent launch: its blocks may be scheduled while that
+// Launches a kernel (in clusters of `cluster` blocks) that depends on the
+// previous one on the stream as a programmatic dependent launch: its blocks may be scheduled while that
 // kernel's last blocks drain, hiding the launch gap; the kernel itself waits
 // (grid_dependency_wait) before touching the results.
 template <class... KArgs, class... Args>
-inline msrep_status launch_dependent(void (*kernel)(KArgs...), int64_t grid, int block,
-                                     cudaStream_t st, size_t smem, Args... args) {
+inline msrep_status launch_dependent_cluster(void (*kernel)(KArgs...), int64_t grid, int block,
+                                             cudaStream_t st, size_t smem, int cluster,
+                                             Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(std::max<int64_t>(grid, 1)));
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   MSREP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
   return MSREP_OK;
+}
+template <class... KArgs, class... Args>
+inline msrep_status launch_dependent(void (*kernel)(KArgs...), int64_t grid, int block,
+                                     cudaStream_t st, size_t smem, Args... args) {
+  return launch_dependent_cluster(kernel, grid, block, st, smem, 1, args...);
+}
+
+// Barrier of all threads of the cluster; what they wrote to global memory
+// before it is visible to all of them after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                   : "memory");
 }
 
 // ---------------------------------------------------------------------------
