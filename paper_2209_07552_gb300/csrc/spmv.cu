@@ -64,12 +64,14 @@ int *kernel_err_ptr() {
 // ---------------------------------------------------------------------------
 
 // Minimum resident blocks per SM asked of the register allocator for the
-// COO direct-load kernel: 3 (80 registers a thread, 24 warps per SM) was
-// measured fastest at the default tile of 512 on GB300 (R-MAT and Laplacian
-// 120 / 114 us; 1 block cap: 125 / 134 us; 4: 127 / 121 us).
-#ifndef MSREP_MINB
-#define MSREP_MINB 3
-#endif
+// row-sorted COO kernel, measured at the default tile of 512 (R-MAT /
+// Laplacian): FP64 108 / 99 us with 3 (80 registers), 114 / 108 with 4, 115 /
+// 113 with 2; FP32 92 / 81, 94 / 79 and 101 / 101; BF16 91 / 85, 88 / 78 and
+// 103 / 110.
+template <class Pol>
+constexpr int coo_blocks() {
+  return sizeof(typename Pol::V) == 2 ? 4 : 3;
+}
 // The same for the CSR kernel: FP64 needs 80 registers (R-MAT / Laplacian 91 /
 // 87 us with 3 blocks, 97 / 90 with 4, which spills); the low-precision forms
 // fit 64 (FP32 71 / 66 us with 4 blocks, 73 / 73 with 3).
@@ -289,7 +291,7 @@ __device__ __forceinline__ void coo_walk(const CooArgs<Pol> &a) {
 }
 
 template <class Pol, int IPT>
-__global__ void __launch_bounds__(kThreads, MSREP_MINB) coo_direct(CooArgs<Pol> a) {
+__global__ void __launch_bounds__(kThreads, coo_blocks<Pol>()) coo_direct(CooArgs<Pol> a) {
   grid_dependency_wait();
   coo_walk(a);
 }
@@ -947,7 +949,7 @@ static msrep_status run_coo(const msrep_matrix *A, const msrep_partition *p,
     return MSREP_OK;
   }
   MSREP_TRY(launch_tiles(coo_stream<Pol, IPT>, coo_direct<Pol, IPT>,
-                         StageGeom<typename Pol::V, IPT, 2>::BLOCK, 0, MSREP_MINB,
+                         StageGeom<typename Pol::V, IPT, 2>::BLOCK, 0, coo_blocks<Pol>(),
                          (flags & MSREP_STREAM_TMA) == 0, T, a.per_part ? p->np : 0, st, a));
   CooTileView v{A->idx2, p->start_idx, p->end_idx, A->nnz, a.G, a.np, A->m};
   int64_t fg = std::min<int64_t>(ceil_div(T, 256), 4 * sm_count());

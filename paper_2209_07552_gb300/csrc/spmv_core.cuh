@@ -686,6 +686,12 @@ __device__ __forceinline__ void coo_tile_range(const CooArgs<Pol> &a, int b, int
   k1 = static_cast<int32_t>(s + (int64_t(g + 1) * L) / a.G);
 }
 
+// A row ends where the next nonzero's row differs, so the loop compares
+// neighbours of the group it holds and finishes the row at its last nonzero.
+// (Finishing it when the next row's first nonzero came up kept the current
+// row in a register and the row-change path, with its empty rows, at every
+// position: R-MAT 2^20 / 2^24 nonzeros FP64 / FP32 116 / 100 us against 108 /
+// 92, Laplacian 110 / 96 against 99 / 81.)
 // kCopy: the caller knows that alpha = 1 and beta = 0, so every row is
 // finished by the copy mode (compile-time: the finishing code shrinks to
 // that case, which keeps the low-precision kernel's loop in the
@@ -725,17 +731,7 @@ __device__ __forceinline__ void coo_tile_compute(const CooArgs<Pol> &a, int b, i
 
   Acc acc = Pol::zero(), first_acc = Pol::zero();
   bool emitted = false;
-  int32_t first_r = 0, cur = -1, lane_next = -1;
-  auto emit = [&]() {
-    if (!emitted) {
-      emitted = true;
-      first_r = cur;
-      first_acc = acc;
-    } else {
-      write_row(cur, acc);
-    }
-    acc = Pol::zero();
-  };
+  int32_t first_r = 0;
   for (int64_t gg = lr.glo; gg < lr.ghi; ++gg) {
     const int64_t g8 = gg << 3;
     int32_t rw[8], c[8];
@@ -744,38 +740,41 @@ __device__ __forceinline__ void coo_tile_compute(const CooArgs<Pol> &a, int b, i
     src.group(row, g8, a.nnz, rw);
     src.group(col, g8, a.nnz, c);
     src.group(val, g8, a.nnz, v);
+    // the row after the group's last nonzero, and past the array's end
+    const int32_t after = g8 + 8 < a.nnz ? __ldg(a.row_idx + g8 + 8) : a.m;
+    if (g8 + 8 > a.nnz) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (g8 + u >= a.nnz) rw[u] = a.m;
+    }
+    const int ulo = static_cast<int>(max(ka - g8, int64_t(0)));
+    const int uhi = static_cast<int>(min(kb - g8, int64_t(8)));
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const bool in = g8 + u >= ka && g8 + u < kb;
+      const bool in = u >= ulo && u < uhi;
       xv[u] = in ? load_x(a.x, c[u]) : typename Pol::X(0);
       if (!in) v[u] = LV(0);
     }
-    const int ulo = static_cast<int>(max(ka - g8, int64_t(0)));
-    const int uhi = static_cast<int>(min(kb - g8, int64_t(8))) - 1;
-    // row of the nonzero right after the lane's range, if it is in this group
-    if (kb < k1 && kb - g8 >= 0 && kb - g8 < 8) lane_next = rw[kb - g8];
-    // row changes branch around FP64-free code; the multiply-adds are the
-    // same instructions on every lane (masked elements add 0)
+    // Row ends branch around FP64-free code; the multiply-adds are the same
+    // instructions on every lane (masked elements add 0).
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      if (u >= ulo && u <= uhi && rw[u] != cur) {
-        if (cur >= 0) {
-          emit();
-          for (int32_t rr = cur + 1; rr < rw[u]; ++rr) write_empty(rr);
-        }
-        cur = rw[u];
-      }
       acc = Pol::template fma<kComp>(acc, v[u], xv[u]);
-    }
-  }
-  // the lane's last run ends here if the next nonzero starts another row
-  if (kb > ka) {
-    int32_t nxt = next_row;
-    if (kb < k1) nxt = (lane_next >= 0) ? lane_next : __ldg(a.row_idx + kb);
-    if (nxt != cur) {
-      emit();
-      if (kb < k1)
-        for (int32_t rr = cur + 1; rr < nxt; ++rr) write_empty(rr);
+      const int32_t next = u < 7 ? rw[u < 7 ? u + 1 : 7] : after;
+      if (u >= ulo && u < uhi && rw[u] != next) {  // a row ends here
+        if (!emitted) {
+          emitted = true;
+          first_r = rw[u];
+          first_acc = acc;
+        } else {
+          write_row(rw[u], acc);
+        }
+        acc = Pol::zero();
+        // rows without nonzeros up to the next one (after the tile's last
+        // nonzero the whole warp fills them, below)
+        if (next - rw[u] > 1 && g8 + u + 1 < k1)
+          for (int32_t rr = rw[u] + 1; rr < next; ++rr) write_empty(rr);
+      }
     }
   }
 
