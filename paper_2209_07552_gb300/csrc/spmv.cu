@@ -6,9 +6,9 @@
 // thread-block tiles (the two-level split of Sec. 4.2, with thread blocks in
 // place of GPUs); tiles never straddle a partition boundary.
 //
-//  CSR  merge-path tiles (rows + nonzeros per tile bounded), per-thread
-//       sequential reduction, block-wide segmented scan, then an
-//       atomic-free fix-up kernel that merges split rows in tile order.
+//  CSR  merge-path tiles (rows + nonzeros per tile bounded), per-lane
+//       sequential reduction, warp segmented scan, then an atomic-free
+//       fix-up that merges split rows in tile order.
 //  COO  nonzero tiles (Alg. 2's split inside each partition), the same
 //       segmented reduction keyed by row_idx, the same fix-up.
 //  CSC  merge-path tiles over col_ptr; each nonzero is scattered into y with

@@ -324,13 +324,7 @@ struct CsrArgs {
   const int32_t *part_toff; // one block per partition: its first tile, or null
 };
 
-template <class Pol>
-__device__ __forceinline__ void write_row(const CsrArgs<Pol> &a, int32_t row,
-                                          typename Pol::Acc v) {
-  a.y[row] = Pol::finish(v, a.finish, a.alpha, a.beta, a.y + row);
-}
-
-// The row pointers of a tile, 32 rows at a time: row i = at() + lane starts
+// The row pointers of a tile, 32 rows at a time: row i = row() starts
 // at start(), ends at end() (valid for i <= nrows; end() for i < nrows only).
 // The first 96 come from registers the caller loaded ahead (p0, p1, p2).
 struct RowChunks {
@@ -356,6 +350,8 @@ struct RowChunks {
   }
 };
 
+// The bulk-copy variant's form of csr_tile (below), which walks the row
+// pointers it has staged; the same sums.
 // One merge-path tile b = rows [r0, r1] x nonzeros [k0, k1), processed by
 // one warp.  rp[j] = row_ptr[r0 + j] for j = 0..r1-r0, and also j = r1-r0+1
 // when r1 < m; rp must be in shared memory (it is searched).
