@@ -501,32 +501,8 @@ __device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32
   tile_k[t] = static_cast<int32_t>(d - r);
 }
 
-// The tile plan of partition i by one warp, for partitions of a few dozen
-// tiles: no search for the partition.
-__device__ __forceinline__ void plan_partition(const int32_t *__restrict__ ptr, int32_t n_major,
-                                               int64_t nnz, int32_t np, const int64_t *D,
-                                               const int32_t *R, const int32_t *tile_off,
-                                               int32_t *tile_row, int32_t *tile_k, int64_t i) {
-  if (i >= np) return;
-  const int lane = threadIdx.x & 31;
-  const int32_t t0 = tile_off[i], t1 = tile_off[i + 1];
-  const int64_t d0 = D[i], len = D[i + 1] - d0;
-  const int32_t lo = R[i], hi = R[i + 1], G = t1 - t0;
-  for (int32_t g = lane; g < G; g += 32) {
-    const int64_t d = d0 + (int64_t(g) * len) / G;
-    const int32_t r = path_row(ptr, lo, hi, d);
-    tile_row[t0 + g] = r;
-    tile_k[t0 + g] = static_cast<int32_t>(d - r);
-  }
-  if (i == np - 1 && lane == 0) {
-    tile_row[t1] = n_major;
-    tile_k[t1] = static_cast<int32_t>(nnz);
-  }
-}
-
 // What the two scans lead to, in one launch: blocks [0, plan_blocks) write
-// the tile plan (a warp per partition, or a thread per tile), the others the
-// local pointers.  A partitioning is a chain of
+// the tile plan, the others the local pointers.  A partitioning is a chain of
 // short dependent launches, so its time is their number times a few
 // microseconds: five took 21.8 us for R-MAT 2^20 / 2^24 nonzeros in 2368
 // partitions with local pointers, three take 15.7.
@@ -534,16 +510,12 @@ template <bool kVec>
 __global__ void __launch_bounds__(256)
     part_fill(const int32_t *__restrict__ ptr, int32_t n_major, int64_t nnz, int32_t np,
               const int64_t *D, const int32_t *R, const int32_t *tile_off, int32_t *tile_row,
-              int32_t *tile_k, int plan_blocks, int by_warp, const int32_t *start_idx,
-              const int32_t *end_idx,
+              int32_t *tile_k, int plan_blocks, const int32_t *start_idx, const int32_t *end_idx,
               const int32_t *start_major, const int32_t *end_major, const int64_t *local_off,
               int32_t *local) {
   grid_dependency_wait();
   const int b = static_cast<int>(blockIdx.x);
-  if (b < plan_blocks && by_warp)
-    plan_partition(ptr, n_major, nnz, np, D, R, tile_off, tile_row, tile_k,
-                   b * int64_t(blockDim.x >> 5) + (threadIdx.x >> 5));
-  else if (b < plan_blocks)
+  if (b < plan_blocks)
     plan_tile(ptr, n_major, nnz, np, D, R, tile_off, tile_row, tile_k,
               b * int64_t(blockDim.x) + threadIdx.x);
   else
@@ -961,13 +933,8 @@ static msrep_status partition_compressed(const msrep_matrix *A,
                                static_cast<const int32_t *>(p->end_major), p->np, p->local_off,
                                static_cast<const int64_t *>(D), tile, toff));
   if (toff || p->local) {
-    // A warp per partition of up to 64 tiles on average (R-MAT, P = 2368: the
-    // search for a tile's partition costs 1.5 us), else a thread per tile
-    // (the one past the last writes the closing entry).  Row blocks can put
-    // most of the tiles into one partition.
-    const int by_warp = L.tmax <= 64 * int64_t(p->np) && !(flags & MSREP_PART_ROW_BLOCK);
-    const int plan_blocks =
-        toff ? static_cast<int>(by_warp ? ceil_div(p->np, 8) : ceil_div(L.tmax + 1, 256)) : 0;
+    // a thread per tile, the one past the last writes the closing entry
+    const int plan_blocks = toff ? static_cast<int>(ceil_div(L.tmax + 1, 256)) : 0;
     // at most m + 2 np local entries (n + 2 np for CSC)
     const int64_t most = int64_t(n_major) + 2 * int64_t(p->np);
     const int fill_blocks =
@@ -981,7 +948,7 @@ static msrep_status partition_compressed(const msrep_matrix *A,
     MSREP_TRY(launch_dependent(fill, plan_blocks + fill_blocks, 256, st, 0, A->ptr, n_major,
                                A->nnz, p->np, static_cast<const int64_t *>(D),
                                static_cast<const int32_t *>(R),
-                               static_cast<const int32_t *>(toff), trow, tk, plan_blocks, by_warp,
+                               static_cast<const int32_t *>(toff), trow, tk, plan_blocks,
                                p->start_idx, p->end_idx, p->start_major, p->end_major,
                                p->local_off, p->local));
   }
