@@ -328,10 +328,17 @@ __global__ void __launch_bounds__(kThreads) coo_stream(CooArgs<Pol> a) {
     fence_mbar_init();
   }
   __syncwarp();
+  // A stage holds a tile of at most 32 * IPT nonzeros.  Equal-nonzero cuts give
+  // no longer one; row blocks (one G for partitions of any length) do, and
+  // such a tile is not staged: it copies nothing (its phase completes at the
+  // arrival) and is read from global memory.
+  auto staged = [](int4 c) { return c.y - c.x <= 32 * IPT; };
   auto plans = [&](int4 c, SegCopy &r, SegCopy &q, SegCopy &v) {
-    r = seg_plan(c.x, c.y, nnz, 4, 8);
-    q = seg_plan(c.x, c.y, nnz, 4, 8);
-    v = seg_plan(c.x, c.y, nnz, sizeof(V), 8);
+    const int32_t end = staged(c) ? c.y : c.x;
+    r = seg_plan(c.x, end, nnz, 4, 8);
+    q = seg_plan(c.x, end, nnz, 4, 8);
+    v = seg_plan(c.x, end, nnz, sizeof(V), 8);
+    if (!staged(c)) r.bytes = q.bytes = v.bytes = 0;
   };
   auto coords = [&](int t) {
     int32_t k0, k1;
@@ -365,15 +372,22 @@ __global__ void __launch_bounds__(kThreads) coo_stream(CooArgs<Pol> a) {
     const int4 c = rec[s];
     SegCopy r, q, v;
     plans(c, r, q, v);
-    const int64_t g_end = min((int64_t(c.y) + 7) & ~int64_t(7), nnz);
-    fill_tail(row_s(s), a.row_idx, r, r.base, g_end);
-    fill_tail(col_s(s), a.col_idx, q, q.base, g_end);
-    fill_tail(val_s(s), a.val, v, v.base, g_end);
-    __syncwarp();
+    if (staged(c)) {  // warp-uniform
+      const int64_t g_end = min((int64_t(c.y) + 7) & ~int64_t(7), nnz);
+      fill_tail(row_s(s), a.row_idx, r, r.base, g_end);
+      fill_tail(col_s(s), a.col_idx, q, q.base, g_end);
+      fill_tail(val_s(s), a.val, v, v.base, g_end);
+      __syncwarp();
+    }
     with_modes<Pol>(kFinishScale, a.comp_mode, [&](auto, auto comp) {
-      coo_tile_compute<Pol, SharedSrc, false, decltype(comp)::value>(
-          a, b, c.x, c.y, Seg<int32_t>{row_s(s), r.base}, Seg<int32_t>{col_s(s), q.base},
-          Seg<V>{val_s(s), v.base}, SharedSrc{});
+      if (staged(c))
+        coo_tile_compute<Pol, SharedSrc, false, decltype(comp)::value>(
+            a, b, c.x, c.y, Seg<int32_t>{row_s(s), r.base}, Seg<int32_t>{col_s(s), q.base},
+            Seg<V>{val_s(s), v.base}, SharedSrc{});
+      else
+        coo_tile_compute<Pol, GlobalSrc, false, decltype(comp)::value>(
+            a, b, c.x, c.y, Seg<int32_t>{a.row_idx, 0}, Seg<int32_t>{a.col_idx, 0},
+            Seg<V>{a.val, 0}, GlobalSrc{});
     });
     __syncwarp();
     if (lane == 0 && b + S * W < T) {
