@@ -394,14 +394,14 @@ msrep_status msrep_autotune(int32_t count, const msrep_matrix *As,
  * a request with 2..8 vectors as one item of the batched k-vector kernel
  * (see msrep_spmm), which reads the matrix once for all its vectors.  Each
  * launch context holds: x and y arenas (arena_bytes each), an interleaved-x
- * arena (4 * arena_bytes), two directories (max_items entries) and tile
+ * arena (4 * arena_bytes), a directory (max_items entries) and tile
  * partials for both kernels (max_tiles and 8 * max_tiles doubles, twice);
  * all of it counts against the budget. */
 typedef struct {
   int64_t budget_bytes;   /* device memory the server may hold in total  */
   int64_t arena_bytes;    /* per in-flight launch: x and y staging (each) */
   int32_t contexts;       /* launches in flight at once (>= 1)           */
-  int32_t max_items;      /* requests per launch, for each kernel        */
+  int32_t max_items;      /* requests per launch                         */
   int32_t max_k;          /* vectors per request (<= 8)                  */
   int32_t tile;           /* tile of every registered matrix (0 = def.)  */
   int64_t max_tiles;      /* tiles per launch, for each kernel           */

@@ -363,12 +363,11 @@ static void scheduler_loop(msrep_server *s) {
         break;
       }
     if (!c) continue;
-    // pack requests in arrival order while the context has room; one-vector
-    // requests fill the SpMV directory, the others the k-vector one
+    // pack requests in arrival order while the context has room: arenas, the
+    // directory (max_items requests) and the partials of either kernel
     std::vector<BatchItem> ritem;
     std::vector<int64_t> rtiles;
     int64_t xf = 0, yf = 0, xtf = 0, tt = 0, ttk = 0;
-    int n1 = 0, nk = 0;
     double bytes = 0;
     c->reqs.clear();
     while (!s->queue.empty()) {
@@ -378,10 +377,11 @@ static void scheduler_loop(msrep_server *s) {
       const int64_t nx = int64_t(R.n) * r->k, ny = int64_t(R.m) * r->k;
       const bool one = r->k == 1;
       const bool full =
-          xf + nx > c->arena_floats || yf + ny > c->arena_floats ||
-          (one ? (n1 + 1 > s->cfg.max_items || tt + R.tiles > c->max_tiles)
-               : (nk + 1 > s->cfg.max_items || ttk + R.tiles > c->max_tiles ||
-                  xtf + int64_t(R.n) * kBatchWidth > c->xt_floats));
+          int64_t(c->reqs.size()) >= s->cfg.max_items || xf + nx > c->arena_floats ||
+          yf + ny > c->arena_floats ||
+          (one ? tt + R.tiles > c->max_tiles
+               : ttk + R.tiles > c->max_tiles ||
+                     xtf + int64_t(R.n) * kBatchWidth > c->xt_floats);
       if (!c->reqs.empty() && full) break;
       s->queue.pop_front();
       c->reqs.push_back(r);
@@ -390,10 +390,8 @@ static void scheduler_loop(msrep_server *s) {
       xf += nx;
       yf += ny;
       if (one) {
-        ++n1;
         tt += R.tiles;
       } else {
-        ++nk;
         ttk += R.tiles;
         xtf += int64_t(R.n) * kBatchWidth;
       }
