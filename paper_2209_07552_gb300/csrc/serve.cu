@@ -468,12 +468,12 @@ static void issuer_loop(msrep_server *s, size_t ci) {
 // list the server's, on every sweep, and the submitting threads waited for
 // both.  A launch whose flag does not come is asked about
 // through its event every kEventPolls sweeps, which is how a failed one shows.
-constexpr int kEventPolls = 4096;
+constexpr uint32_t kEventPolls = 4096;
 static void completion_loop(msrep_server *s) {
   cudaSetDevice(s->cfg.device);
   std::vector<Context *> flying;
   uint64_t seen = 0;
-  int sweeps = 0;
+  uint32_t sweeps = 0;  // wraps
   for (;;) {
     if (flying.empty() || s->issued.load() != seen) {
       std::unique_lock<std::mutex> lk(s->mu);
