@@ -37,7 +37,7 @@ msrep_status launch_batched(const BatchItem *items, const int64_t *toff, int cou
                             int64_t total_tiles, int32_t val_dtype, const void *const *xs,
                             void *const *ys, double *head, double *tail, double alpha,
                             double beta, unsigned flags, cudaStream_t st,
-                            int cta_threads = 256, int max_tile = 1024);
+                            int cta_threads, int max_tile);
 
 // Batched k-vector form (FP32 values and vectors): item j carries
 // 2 <= k_j <= 8 vectors, xin[j] = its k_j x vectors of n_j values each

@@ -173,6 +173,8 @@ __global__ void serve_signal(volatile uint32_t *flag, uint32_t number) {
   *flag = number;
 }
 
+constexpr int kServeThreads = 256;  // of the batched SpMV kernel's blocks
+
 static msrep_status launch_copies(const CopyItem *items, int count, cudaStream_t st) {
   if (count == 0) return MSREP_OK;
   serve_copy<<<dim3(32, std::min(count, 1024)), 256, 0, st>>>(items, count);
@@ -320,7 +322,7 @@ static msrep_status launch_context(msrep_server *s, Context &c,
                              reinterpret_cast<const int64_t *>(dd + L.toff), n1, tt, MSREP_F32,
                              reinterpret_cast<const void *const *>(dd + L.xs),
                              reinterpret_cast<void *const *>(dd + L.ys), c.head, c.tail, 1.0, 0.0,
-                             0, c.stream));
+                             0, c.stream, kServeThreads, effective_tile(s->cfg.tile)));
   if (nk > 0)
     MSREP_TRY(launch_batched_k(reinterpret_cast<const BatchItem *>(dd + L.itk),
                                reinterpret_cast<const int64_t *>(dd + L.toffk),
