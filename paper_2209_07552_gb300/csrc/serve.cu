@@ -8,8 +8,9 @@
 // queued requests into a launch whenever a context (stream + x/y arenas +
 // directory buffers) is free and hands it to the context's own issuing
 // thread, which issues its copies and kernels (so that the issuing of
-// several launches overlaps); a completion thread polls each context's
-// event, copies y back to the callers' buffers and wakes the waiters.
+// several launches overlaps); a completion thread watches a host flag that
+// each context's launch sets at its end, copies staged y to the callers'
+// buffers and wakes the waiters.
 // Several contexts are in flight at once, so requests that arrive while
 // others run are admitted as soon as a context frees up, and their work
 // overlaps on the device.
@@ -175,6 +176,16 @@ __global__ void serve_signal(volatile uint32_t *flag, uint32_t number) {
 
 constexpr int kServeThreads = 256;  // of the batched SpMV kernel's blocks
 
+// A y of at least this many vectors and bytes is copied out after the kernels:
+// the k-vector kernel's own writes to host memory then hold its 16 warps an SM
+// up for longer than the copy takes.  One request of 8 / 4 vectors, 2^20 rows
+// of a Laplacian: 491 / 294 us copied out, 576 / 318 written directly; of 50,000
+// rows 93 / 81 and 93 / 79, of 1,000 rows 71 / 69 and 67 / 64.  Of 3, 2 or 1
+// vectors, R-MAT 2^20 rows: 309, 253, 152 us copied out, 284, 234, 140 written
+// directly.
+constexpr int kCopyOutVectors = 4;
+constexpr int64_t kCopyOutBytes = int64_t(2) << 20;
+
 static msrep_status launch_copies(const CopyItem *items, int count, cudaStream_t st) {
   if (count == 0) return MSREP_OK;
   serve_copy<<<dim3(32, std::min(count, 1024)), 256, 0, st>>>(items, count);
@@ -206,8 +217,8 @@ static void free_context(Context &c) {
 
 // Per-launch directory, laid out for the launch's R requests (so that one
 // copy of about 250 bytes a request carries it): the SpMV items (one-vector
-// requests) with their tile offsets and x / y pointers, the copy list (x in),
-// and the k-vector items with tile and unit offsets and
+// requests) with their tile offsets and x / y pointers, the copy list (x in, y
+// out), and the k-vector items with tile and unit offsets and
 // their x / interleaved-x / y pointers.
 struct LaunchDir {
   size_t items, toff, xs, ys, cin, itk, toffk, uoffk, xin, xtp, ysk, bytes;
@@ -243,7 +254,8 @@ static size_t dir_size(int32_t max_items) { return LaunchDir(size_t(max_items)).
 // SpMV gathers it at random), x of a k-vector request is read by the
 // interleaving kernel itself, and a mapped y is written by the SpMV kernels
 // as they finish its rows, once each, so its way over the host link overlaps
-// their work.  A pageable y is written to the pinned staging arena in the same
+// their work, unless it is large and holds many vectors (kCopyOut*): those are
+// written to the arena and copied out by one copy kernel.  A pageable y is written to the pinned staging arena in the same
 // way (copied there by DMA, the launch's end waited for the copy engine to hand
 // over to the signalling kernel: a request of 1,000 rows took 72 us, not 62).
 // Other buffers take one DMA copy each (a pageable x staged through the pinned
@@ -259,7 +271,9 @@ static msrep_status launch_context(msrep_server *s, Context &c,
   int64_t *toff = reinterpret_cast<int64_t *>(dp + L.toff);
   const void **xs = reinterpret_cast<const void **>(dp + L.xs);
   void **ys = reinterpret_cast<void **>(dp + L.ys);
-  CopyItem *cin = reinterpret_cast<CopyItem *>(dp + L.cin);
+  // one list: x of one-vector requests from the front, y of k-vector ones from
+  // the back
+  CopyItem *cin = reinterpret_cast<CopyItem *>(dp + L.cin), *cout = cin + R;
   BatchItem *itk = reinterpret_cast<BatchItem *>(dp + L.itk);
   int64_t *toffk = reinterpret_cast<int64_t *>(dp + L.toffk);
   int64_t *uoffk = reinterpret_cast<int64_t *>(dp + L.uoffk);
@@ -268,7 +282,7 @@ static msrep_status launch_context(msrep_server *s, Context &c,
   void **ysk = reinterpret_cast<void **>(dp + L.ysk);
 
   int64_t xo = 0, yo = 0, xto = 0, tt = 0, ttk = 0, utk = 0;
-  int n1 = 0, nk = 0, nci = 0;
+  int n1 = 0, nk = 0, nci = 0, nco = 0;
   c.y_off.clear();
   MSREP_CUDA_TRY(cudaEventRecord(c.begin_ev, c.stream));
   for (size_t i = 0; i < R; ++i) {
@@ -289,7 +303,12 @@ static msrep_status launch_context(msrep_server *s, Context &c,
       MSREP_CUDA_TRY(cudaMemcpyAsync(c.x_dev + xo, c.x_pin + xo, xb, cudaMemcpyHostToDevice, c.stream));
     }
     float *yhost = r->y_map ? r->y_map : r->y_pinned ? nullptr : c.y_pin + yo;
+    const int64_t ny = int64_t(bi.m) * r->k;
     float *ydst = yhost ? yhost : c.y_dev + yo;  // where they write its y
+    if (yhost && r->k >= kCopyOutVectors && int64_t(sizeof(float)) * ny >= kCopyOutBytes) {
+      ydst = c.y_dev + yo;
+      cout[-++nco] = CopyItem{ydst, yhost, ny};
+    }
     if (r->k == 1) {
       it[n1] = bi;
       toff[n1] = tt;
@@ -311,7 +330,7 @@ static msrep_status launch_context(msrep_server *s, Context &c,
       ++nk;
     }
     xo += nx;
-    yo += int64_t(bi.m) * r->k;
+    yo += ny;
   }
   toff[n1] = tt;
   toffk[nk] = ttk;
@@ -335,6 +354,8 @@ static msrep_status launch_context(msrep_server *s, Context &c,
                                reinterpret_cast<void *const *>(dd + L.ysk), c.head_k, c.tail_k, 0,
                                c.stream));
   MSREP_CUDA_TRY(cudaEventRecord(c.k1_ev, c.stream));
+  MSREP_TRY(launch_copies(reinterpret_cast<const CopyItem *>(dd + L.cin) + (R - nco), nco,
+                          c.stream));
   for (size_t i = 0; i < R; ++i) {
     const auto &r = c.reqs[i];
     if (r->y_map || !r->y_pinned) continue;
