@@ -52,29 +52,33 @@ int sm_count() {
 // searches over a compressed pointer array
 // ---------------------------------------------------------------------------
 
-// Largest r in [lo, hi] with ptr[r] <= k (the row owning nonzero k), found
+// Largest r in [lo, hi] with at(r) <= k, at non-decreasing (of a pointer array:
+// the row owning nonzero k), found
 // by a whole warp: each round the 32 lanes probe 32 evenly spaced points of
 // [lo, hi] and the range shrinks about 33-fold (about five dependent loads
 // for a million rows instead of twenty for a binary search).  Every lane
-// returns the result.  Requires ptr[lo] <= k.
-template <typename T>
-__device__ __forceinline__ int32_t last_le_warp(const T *__restrict__ ptr, int32_t lo,
-                                                int32_t hi, int64_t k) {
+// returns the result.  Requires at(lo) <= k.
+template <class At>
+__device__ __forceinline__ int32_t last_le_warp_at(At at, int32_t lo, int32_t hi, int64_t k) {
   const int lane = threadIdx.x & 31;
   while (hi - lo >= 32) {
     const int64_t span = int64_t(hi) - lo;
     const int32_t q = lo + static_cast<int32_t>((int64_t(lane) + 1) * span / 33);
-    const bool le = static_cast<int64_t>(__ldg(ptr + q)) <= k;
-    // ptr is non-decreasing and q increases with the lane: the lanes with
-    // ptr[q] <= k form a prefix
+    const bool le = at(q) <= k;
+    // the values are non-decreasing and q increases with the lane: the lanes
+    // with at(q) <= k form a prefix
     const int t = __popc(__ballot_sync(0xffffffffu, le));
     const int32_t qlo = __shfl_sync(0xffffffffu, q, t > 0 ? t - 1 : 0);
     const int32_t qhi = __shfl_sync(0xffffffffu, q, t < 32 ? t : 31);
     if (t > 0) lo = qlo;
     if (t < 32) hi = qhi - 1;
   }
-  const bool le = lo + lane <= hi && static_cast<int64_t>(__ldg(ptr + lo + lane)) <= k;
+  const bool le = lo + lane <= hi && at(lo + lane) <= k;
   return lo + __popc(__ballot_sync(0xffffffffu, le)) - 1;
+}
+__device__ __forceinline__ int32_t last_le_warp(const int32_t *__restrict__ ptr, int32_t lo,
+                                                int32_t hi, int64_t k) {
+  return last_le_warp_at([ptr](int32_t q) { return int64_t(__ldg(ptr + q)); }, lo, hi, k);
 }
 
 // last_le_warp on the merge path: largest r in [lo, hi] with
@@ -310,7 +314,71 @@ __device__ T block_exclusive_scan(T v, T &total) {
   return base + inc - v;
 }
 
-// The two scans over partitions (CSR/CSC), a block each: local_off[i] =
+// The lengths the two offset arrays sum up: entries of partition i's local
+// pointers, and its tiles (a tile is a power of two).
+struct LocalLen {
+  const int32_t *start_major, *end_major;
+  __device__ __forceinline__ int64_t operator()(int32_t i) const {
+    return int64_t(end_major[i]) - start_major[i] + 2;
+  }
+};
+struct TileLen {
+  const int64_t *D;
+  int32_t tile;
+  __device__ __forceinline__ int64_t operator()(int32_t i) const {
+    return (D[i + 1] - D[i] + tile - 1) >> __popc(tile - 1);
+  }
+};
+
+// Offsets of at most kScanMax partitions: s_off[i] = sum_{j<i} len(j), i <= np,
+// in shared memory, by a block of kFillThreads.  A warp takes a stretch of
+// partitions, 32 at a time; its loads are all in flight at once.  The sums fit
+// 32 bits: at most 2^31 + 2 np local entries, and fewer tiles.
+constexpr int kFillThreads = 256;
+constexpr int kScanMax = 4096;
+template <class Len>
+__device__ __forceinline__ void block_offsets(int32_t np, Len len, uint32_t *s_off) {
+  constexpr int kWarps = kFillThreads / 32, kRows = kScanMax / kFillThreads;
+  __shared__ uint32_t s_warp[kWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int rows = (np + kFillThreads - 1) / kFillThreads, first = wid * rows * 32 + lane;
+  uint32_t g[kRows];
+#pragma unroll
+  for (int j = 0; j < kRows; ++j) {
+    const int i = first + 32 * j;
+    g[j] = j < rows && i < np ? static_cast<uint32_t>(len(i)) : 0u;
+  }
+  uint32_t sum = 0;
+#pragma unroll
+  for (int j = 0; j < kRows; ++j)
+    if (j < rows) {
+      uint32_t inc = g[j];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+      }
+      g[j] = sum + inc - g[j];
+      sum += __shfl_sync(0xffffffffu, inc, 31);
+    }
+  if (lane == 0) s_warp[wid] = sum;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    if (w < wid) before += s_warp[w];
+    total += s_warp[w];
+  }
+#pragma unroll
+  for (int j = 0; j < kRows; ++j) {
+    const int i = first + 32 * j;
+    if (j < rows && i < np) s_off[i] = before + g[j];
+  }
+  if (threadIdx.x == 0) s_off[np] = total;
+  __syncthreads();
+}
+
+// The same for any number of partitions, a block for each array: local_off[i] =
 // sum_{j<i} (end_major[j] - start_major[j] + 2), and the tile plan's first
 // tiles, tile_off[i] = sum_{j<i} ceil((D[j+1] - D[j]) / tile).  Either array
 // may be null (not wanted); block 0 takes the first one wanted.
@@ -324,8 +392,7 @@ __global__ void __launch_bounds__(1024)
     const int32_t i = base + threadIdx.x;
     int64_t len = 0;
     if (i < np)
-      len = tiles ? (D[i + 1] - D[i] + tile - 1) / tile
-                  : int64_t(end_major[i]) - start_major[i] + 2;
+      len = tiles ? TileLen{D, tile}(i) : LocalLen{start_major, end_major}(i);
     int64_t total;
     const int64_t ex = block_exclusive_scan<int64_t>(len, total);
     if (i < np) {
@@ -353,29 +420,31 @@ __global__ void __launch_bounds__(1024)
 // partitions' row spans are.  Entry j of partition i: 0 (j = 0),
 // end - start + 1 (j = span + 1), else ptr[start_major + j] - start_idx.
 // Block `block` of `blocks`.
-template <bool kVec>
+// off(i): the offset of partition i, i <= np.
+template <bool kVec, class Off>
 __device__ __forceinline__ void
     local_fill_compressed(const int32_t *__restrict__ ptr, const int32_t *start_idx,
                           const int32_t *end_idx, const int32_t *start_major,
-                          const int32_t *end_major, const int64_t *local_off, int32_t np,
+                          const int32_t *end_major, Off off, int32_t np,
                           int32_t *local, int block, int blocks) {
-  const int64_t total = local_off[np];
+  const int64_t total = off(np);
   const int lane = threadIdx.x & 31;
   const int64_t warps = int64_t(blocks) * (blockDim.x >> 5);
   for (int64_t w0 = (block * int64_t(blockDim.x >> 5) + (threadIdx.x >> 5)) * 256;
        w0 < total; w0 += warps * 256) {
     // partitions of the warp's first and last entries (warp-uniform)
-    const int32_t ia = last_le_warp(local_off, 0, np - 1, w0);
-    const int32_t ib = last_le_warp(local_off, ia, np - 1, w0 + 255 < total ? w0 + 255 : total - 1);
+    const int32_t ia = last_le_warp_at(off, 0, np - 1, w0);
+    const int32_t ib =
+        last_le_warp_at(off, ia, np - 1, w0 + 255 < total ? w0 + 255 : total - 1);
     const int64_t t0 = w0 + 8 * lane;
     if (t0 >= total) continue;
-    int32_t lo = ia, hi = ib;  // last i in [ia, ib] with local_off[i] <= t0
+    int32_t lo = ia, hi = ib;  // last i in [ia, ib] with off(i) <= t0
     while (lo < hi) {
       const int32_t mid = (lo + hi + 1) >> 1;
-      if (__ldg(local_off + mid) <= t0) lo = mid; else hi = mid - 1;
+      if (off(mid) <= t0) lo = mid; else hi = mid - 1;
     }
     int32_t i = lo;
-    int64_t base = __ldg(local_off + i), next = __ldg(local_off + i + 1);
+    int64_t base = off(i), next = off(i + 1);
     int32_t sm = __ldg(start_major + i), span = __ldg(end_major + i) - sm;
     int32_t s = __ldg(start_idx + i), e = __ldg(end_idx + i);
     int32_t v[8];
@@ -385,7 +454,7 @@ __device__ __forceinline__ void
       while (t >= next && i + 1 < np) {
         ++i;
         base = next;
-        next = __ldg(local_off + i + 1);
+        next = off(i + 1);
         sm = __ldg(start_major + i);
         span = __ldg(end_major + i) - sm;
         s = __ldg(start_idx + i);
@@ -470,15 +539,16 @@ __global__ void __launch_bounds__(256)
 // [D_i, D_{i+1}) is split into ceil(len / tile) equal pieces
 // ---------------------------------------------------------------------------
 
-// A thread per tile t: its partition is the last i with tile_off[i] <= t (a
+// A thread per tile t: its partition is the last i with off(i) <= t (a
 // partition without tiles shares its offset with the next), its diagonal the
 // g-th even cut of that partition's stretch.  (A block per partition left a
 // matrix in one partition to 128 threads: 462 us for 2^24 nonzeros.)
+template <class Off>
 __device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32_t n_major,
                                           int64_t nnz, int32_t np, const int64_t *D,
-                                          const int32_t *R, const int32_t *tile_off,
-                                          int32_t *tile_row, int32_t *tile_k, int64_t t) {
-  const int32_t T = tile_off[np];
+                                          const int32_t *R, Off off, int32_t *tile_row,
+                                          int32_t *tile_k, int64_t t) {
+  const int64_t T = off(np);
   if (t > T) return;
   if (t == T) {
     tile_row[T] = n_major;
@@ -488,12 +558,12 @@ __device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32
   int32_t lo = 0, hi = np - 1;
   while (lo < hi) {
     const int32_t mid = lo + (hi - lo + 1) / 2;
-    if (__ldg(tile_off + mid) <= t)
+    if (off(mid) <= t)
       lo = mid;
     else
       hi = mid - 1;
   }
-  const int32_t t0 = __ldg(tile_off + lo), G = __ldg(tile_off + lo + 1) - t0;
+  const int64_t t0 = off(lo), G = off(lo + 1) - t0;
   const int64_t d0 = __ldg(D + lo), len = __ldg(D + lo + 1) - d0;
   const int64_t d = d0 + ((t - t0) * len) / G;
   const int32_t r = path_row(ptr, __ldg(R + lo), __ldg(R + lo + 1), d);
@@ -501,26 +571,55 @@ __device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32
   tile_k[t] = static_cast<int32_t>(d - r);
 }
 
-// What the two scans lead to, in one launch: blocks [0, plan_blocks) write
-// the tile plan, the others the local pointers.  A partitioning is a chain of
-// short dependent launches, so its time is their number times a few
-// microseconds: five took 21.8 us for R-MAT 2^20 / 2^24 nonzeros in 2368
-// partitions with local pointers, three take 15.7.
-template <bool kVec>
-__global__ void __launch_bounds__(256)
+// The offsets and what they lead to: blocks [0, plan_blocks) write the tile
+// plan, the others the local pointers (local may be null: offsets alone).  A
+// partitioning is a chain of short dependent launches, so its time is their
+// number, and the dependent loads in each, times a microsecond or so.
+// kScan: every block sums the lengths of all partitions itself, which takes
+// less than a launch between, and searches them in shared memory instead of a
+// dependent load per bit of np; the first block of each kind writes the offsets
+// out.  Otherwise part_scans has written them.  R-MAT 2^20 / 2^24 nonzeros, the
+// plan alone, 592 and 2368 partitions: 10.3 and 12.5 us, 12.9 and 14.6 with
+// part_scans; 2368 with local pointers 13.5 and 16.4.
+template <bool kVec, bool kScan>
+__global__ void __launch_bounds__(kFillThreads)
     part_fill(const int32_t *__restrict__ ptr, int32_t n_major, int64_t nnz, int32_t np,
-              const int64_t *D, const int32_t *R, const int32_t *tile_off, int32_t *tile_row,
-              int32_t *tile_k, int plan_blocks, const int32_t *start_idx, const int32_t *end_idx,
-              const int32_t *start_major, const int32_t *end_major, const int64_t *local_off,
-              int32_t *local) {
+              const int64_t *D, const int32_t *R, int32_t tile, int32_t *tile_off,
+              int32_t *tile_row, int32_t *tile_k, int plan_blocks, const int32_t *start_idx,
+              const int32_t *end_idx, const int32_t *start_major, const int32_t *end_major,
+              int64_t *local_off, int32_t *local) {
+  __shared__ uint32_t s_off[kScan ? kScanMax + 1 : 1];
   grid_dependency_wait();
   const int b = static_cast<int>(blockIdx.x);
-  if (b < plan_blocks)
-    plan_tile(ptr, n_major, nnz, np, D, R, tile_off, tile_row, tile_k,
-              b * int64_t(blockDim.x) + threadIdx.x);
-  else
-    local_fill_compressed<kVec>(ptr, start_idx, end_idx, start_major, end_major, local_off, np,
-                                local, b - plan_blocks, static_cast<int>(gridDim.x) - plan_blocks);
+  auto shared_off = [&](int32_t i) { return int64_t(s_off[i]); };
+  if (b < plan_blocks) {
+    const int64_t t = b * int64_t(kFillThreads) + threadIdx.x;
+    if constexpr (kScan) {
+      block_offsets(np, TileLen{D, tile}, s_off);
+      if (b == 0)
+        for (int32_t i = threadIdx.x; i <= np; i += kFillThreads)
+          tile_off[i] = static_cast<int32_t>(s_off[i]);
+      plan_tile(ptr, n_major, nnz, np, D, R, shared_off, tile_row, tile_k, t);
+    } else {
+      plan_tile(ptr, n_major, nnz, np, D, R,
+                [tile_off](int32_t i) { return int64_t(__ldg(tile_off + i)); }, tile_row, tile_k,
+                t);
+    }
+  } else {
+    const int block = b - plan_blocks, blocks = static_cast<int>(gridDim.x) - plan_blocks;
+    if constexpr (kScan) {
+      block_offsets(np, LocalLen{start_major, end_major}, s_off);
+      if (block == 0)
+        for (int32_t i = threadIdx.x; i <= np; i += kFillThreads) local_off[i] = s_off[i];
+      if (local)
+        local_fill_compressed<kVec>(ptr, start_idx, end_idx, start_major, end_major, shared_off,
+                                    np, local, block, blocks);
+    } else if (local) {
+      local_fill_compressed<kVec>(ptr, start_idx, end_idx, start_major, end_major,
+                                  [local_off](int32_t i) { return __ldg(local_off + i); }, np,
+                                  local, block, blocks);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -927,28 +1026,33 @@ static msrep_status partition_compressed(const msrep_matrix *A,
                                       : (flags & MSREP_PART_ROW_BLOCK) ? int(kCutRowBlock)
                                                                        : int(kCutNonzeros)));
   int32_t *toff = plan ? reinterpret_cast<int32_t *>(plan + L.off_toff) : nullptr;
-  if (toff || p->local_off)
+  // a thread per tile, the one past the last writes the closing entry
+  const int plan_blocks = toff ? static_cast<int>(ceil_div(L.tmax + 1, kFillThreads)) : 0;
+  // at most m + 2 np local entries (n + 2 np for CSC)
+  const int64_t most = int64_t(n_major) + 2 * int64_t(p->np);
+  const int fill_blocks =
+      p->local ? static_cast<int>(std::max<int64_t>(
+                     1, std::min<int64_t>(ceil_div(most, 8 * 256), 8 * sm_count())))
+               : p->local_off ? 1 : 0;
+  // Every block scans (part_fill) where that takes less than a launch: up to
+  // 4096 partitions (R-MAT plan alone, 8192: 24.7 us against 22.8), and four
+  // blocks of local pointers an SM (R-MAT, 515 of them: 13.5 us against 16.4;
+  // Laplacian 2048^2, 1216: 23.6 against 21.8)
+  const bool scan = p->np <= kScanMax && fill_blocks <= 4 * sm_count();
+  if (!scan && (toff || p->local_off))
     MSREP_TRY(launch_dependent(part_scans, toff && p->local_off ? 2 : 1, 1024, st, 0,
                                static_cast<const int32_t *>(p->start_major),
                                static_cast<const int32_t *>(p->end_major), p->np, p->local_off,
                                static_cast<const int64_t *>(D), tile, toff));
-  if (toff || p->local) {
-    // a thread per tile, the one past the last writes the closing entry
-    const int plan_blocks = toff ? static_cast<int>(ceil_div(L.tmax + 1, 256)) : 0;
-    // at most m + 2 np local entries (n + 2 np for CSC)
-    const int64_t most = int64_t(n_major) + 2 * int64_t(p->np);
-    const int fill_blocks =
-        p->local ? static_cast<int>(std::max<int64_t>(
-                       1, std::min<int64_t>(ceil_div(most, 8 * 256), 8 * sm_count())))
-                 : 0;
-    const auto fill = (reinterpret_cast<uintptr_t>(p->local) & 15) == 0 ? part_fill<true>
-                                                                        : part_fill<false>;
+  if (toff || p->local || (scan && p->local_off)) {
+    const bool vec = (reinterpret_cast<uintptr_t>(p->local) & 15) == 0;
+    const auto fill = scan ? (vec ? part_fill<true, true> : part_fill<false, true>)
+                           : (vec ? part_fill<true, false> : part_fill<false, false>);
     int32_t *trow = plan ? reinterpret_cast<int32_t *>(plan + L.off_row) : nullptr;
     int32_t *tk = plan ? reinterpret_cast<int32_t *>(plan + L.off_k) : nullptr;
-    MSREP_TRY(launch_dependent(fill, plan_blocks + fill_blocks, 256, st, 0, A->ptr, n_major,
-                               A->nnz, p->np, static_cast<const int64_t *>(D),
-                               static_cast<const int32_t *>(R),
-                               static_cast<const int32_t *>(toff), trow, tk, plan_blocks,
+    MSREP_TRY(launch_dependent(fill, plan_blocks + fill_blocks, kFillThreads, st, 0, A->ptr,
+                               n_major, A->nnz, p->np, static_cast<const int64_t *>(D),
+                               static_cast<const int32_t *>(R), tile, toff, trow, tk, plan_blocks,
                                p->start_idx, p->end_idx, p->start_major, p->end_major,
                                p->local_off, p->local));
   }
