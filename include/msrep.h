@@ -294,7 +294,8 @@ msrep_status msrep_spmm_workspace_size(const msrep_matrix *A, const msrep_partit
  * MSREP_SPMM_MAX_K (8): each pass first copies its vectors into the
  * workspace with their values of each row side by side, so that each
  * nonzero gathers one segment for all of them and A is read once per pass
- * (ceil(k / 8) times in all).  Every column of Y is computed exactly as
+ * (ceil(k / 8) times in all).  A pass of one vector is msrep_spmv's, on x in
+ * place or, where y overlaps it, on its copy.  Every column of Y is computed exactly as
  * msrep_spmv computes y for that x (same order of operations,
  * bit-identical results).  `flags`: MSREP_COMP_ALL / MSREP_COMP_NONE as
  * for msrep_spmv.  Asynchronous on `stream`.

@@ -17,6 +17,9 @@ namespace msrep {
 
 msrep_status check_matrix(const msrep_matrix *A);
 int32_t effective_tile(int32_t tile);
+msrep_status spmv_csr_tiles(const msrep_matrix *A, const msrep_partition *p, double alpha,
+                            const void *x, double beta, void *y, unsigned flags, double *head,
+                            double *tail, cudaStream_t st);
 
 // xt[c * KP + j] = x[j * ldx + c] for j < k, 0 for k <= j < KP; a thread
 // per column: coalesced reads of each vector, the row written as 16-byte
@@ -168,12 +171,33 @@ static msrep_status run_spmm(const msrep_matrix *A, const msrep_partition *p, in
   return MSREP_OK;
 }
 
+// One vector: the SpMV kernels, which have no row buffer to fill and finish
+// small problems in one launch.  They read x where it lies, unless y overlaps
+// it: then, as with more vectors, its copy in the workspace.
+template <class X>
+static msrep_status run_one(const msrep_matrix *A, const msrep_partition *p, double alpha,
+                            const void *x, double beta, void *y, unsigned flags, void *ws,
+                            cudaStream_t st) {
+  const PlanLayout L = plan_layout(A->m, A->nnz, p->np, effective_tile(p->tile));
+  double *head = nullptr, *tail = nullptr;
+  void *xt = nullptr;
+  spmm_ws_layout(L.tmax, 1, A->n, sizeof(X), &head, &tail, &xt, ws);
+  const uintptr_t x0 = reinterpret_cast<uintptr_t>(x), y0 = reinterpret_cast<uintptr_t>(y);
+  if (x0 < y0 + sizeof(X) * size_t(A->m) && y0 < x0 + sizeof(X) * size_t(A->n)) {
+    MSREP_TRY(launch_dependent(interleave_x<X, 1>, 4 * sm_count(), 256, st, 0,
+                               static_cast<const X *>(x), A->n, 1, A->n, static_cast<X *>(xt)));
+    x = xt;
+  }
+  return spmv_csr_tiles(A, p, alpha, x, beta, y, flags & (MSREP_COMP_ALL | MSREP_COMP_NONE), head,
+                        tail, st);
+}
+
 template <class Pol>
 static msrep_status dispatch_k(const msrep_matrix *A, const msrep_partition *p, int k,
                                double alpha, const void *x, int64_t ldx, double beta, void *y,
                                int64_t ldy, unsigned flags, void *ws, cudaStream_t st) {
   switch (spmm_width(k)) {
-    case 1: return run_spmm<Pol, 1>(A, p, k, alpha, x, ldx, beta, y, ldy, flags, ws, st);
+    case 1: return run_one<typename Pol::X>(A, p, alpha, x, beta, y, flags, ws, st);
     case 2: return run_spmm<Pol, 2>(A, p, k, alpha, x, ldx, beta, y, ldy, flags, ws, st);
     case 4: return run_spmm<Pol, 4>(A, p, k, alpha, x, ldx, beta, y, ldy, flags, ws, st);
     default: return run_spmm<Pol, 8>(A, p, k, alpha, x, ldx, beta, y, ldy, flags, ws, st);

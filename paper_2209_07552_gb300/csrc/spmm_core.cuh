@@ -142,14 +142,8 @@ struct KvAcc<PolF64, VW> {
   double a[VW];
   struct XV {
     double d[VW];
-    __device__ __forceinline__ void zero() {
-#pragma unroll
-      for (int j = 0; j < VW; ++j) d[j] = 0.0;
-    }
     __device__ __forceinline__ void load(const double *p) {
-      if constexpr (VW == 1) {
-        d[0] = __ldg(p);
-      } else if constexpr (VW == 2) {
+      if constexpr (VW == 2) {
         const double2 t = __ldg(reinterpret_cast<const double2 *>(p));
         d[0] = t.x;
         d[1] = t.y;
@@ -171,24 +165,16 @@ struct KvAcc<PolF64, VW> {
     for (int j = 0; j < VW; ++j) a[j] = __fma_rn(v, x.d[j], a[j]);
   }
   __device__ __forceinline__ void store(double *p) const {
-    if constexpr (VW == 1) {
-      p[0] = a[0];
-    } else {
 #pragma unroll
-      for (int j = 0; j < VW; j += 2)
-        *reinterpret_cast<double2 *>(p + j) = make_double2(a[j], a[j + 1]);
-    }
+    for (int j = 0; j < VW; j += 2)
+      *reinterpret_cast<double2 *>(p + j) = make_double2(a[j], a[j + 1]);
   }
   __device__ __forceinline__ void load(const double *p) {
-    if constexpr (VW == 1) {
-      a[0] = p[0];
-    } else {
 #pragma unroll
-      for (int j = 0; j < VW; j += 2) {
-        const double2 t = *reinterpret_cast<const double2 *>(p + j);
-        a[j] = t.x;
-        a[j + 1] = t.y;
-      }
+    for (int j = 0; j < VW; j += 2) {
+      const double2 t = *reinterpret_cast<const double2 *>(p + j);
+      a[j] = t.x;
+      a[j + 1] = t.y;
     }
   }
   __device__ __forceinline__ void totals(double (&t)[VW]) const {
@@ -219,10 +205,6 @@ struct KvAcc<PolF32<VT>, VW> {
   f32x2 s[N2], c[N2];
   struct XV {
     f32x2 d[N2];
-    __device__ __forceinline__ void zero() {
-#pragma unroll
-      for (int j = 0; j < N2; ++j) d[j] = 0;
-    }
     __device__ __forceinline__ void load(const float *p) {
       if constexpr (VW == 2) {
         asm("ld.global.nc.b64 %0, [%1];" : "=l"(d[0]) : "l"(p));
@@ -316,36 +298,6 @@ struct KvAcc<PolF32<VT>, VW> {
       r.s[j] = __shfl_up_sync(0xffffffffu, s[j], o);
       r.c[j] = __shfl_up_sync(0xffffffffu, c[j], o);
     }
-    return r;
-  }
-};
-
-// one FP32 vector
-template <class VT>
-struct KvAcc<PolF32<VT>, 1> {
-  using X = float;
-  using Pol = PolF32<VT>;
-  F32Pair a;
-  struct XV {
-    float d;
-    __device__ __forceinline__ void zero() { d = 0.f; }
-    __device__ __forceinline__ void load(const float *p) { d = __ldg(p); }
-  };
-  __device__ __forceinline__ void zero() { a = Pol::zero(); }
-  template <bool kComp>
-  __device__ __forceinline__ void fma(float v, const XV &x) {
-    a = Pol::template fma<kComp>(a, v, x.d);
-  }
-  __device__ __forceinline__ void store(float *p) const {
-    p[0] = a.s;
-    p[1] = a.c;
-  }
-  __device__ __forceinline__ void load(const float *p) { a = F32Pair{p[0], p[1]}; }
-  __device__ __forceinline__ void totals(float (&t)[1]) const { t[0] = pair_total(a.s, a.c); }
-  __device__ __forceinline__ void carry_in(const KvAcc &u) { a = Pol::combine(u.a, a); }
-  __device__ __forceinline__ KvAcc shfl_up(int o) const {
-    KvAcc r;
-    r.a = Pol::shfl_up(a, o);
     return r;
   }
 };

@@ -1113,6 +1113,31 @@ static msrep_status dispatch_tile(const msrep_matrix *A, const msrep_partition *
   return fail(MSREP_ERR_INVALID_ARG, "unsupported tile %d", tile);
 }
 
+// CSR over the plan's tiles with the caller's partials (head, tail: the plan's
+// tile bound of doubles each): msrep_spmm's form for one vector.
+msrep_status spmv_csr_tiles(const msrep_matrix *A, const msrep_partition *p, double alpha,
+                            const void *x, double beta, void *y, unsigned flags, double *head,
+                            double *tail, cudaStream_t st) {
+  Workspace w;
+  w.head = head;
+  w.tail = tail;
+  w.yacc = nullptr;
+  w.perm = false;
+  auto run = [&](auto pol) -> msrep_status {
+    using Pol = decltype(pol);
+    switch (effective_tile(p->tile)) {
+      case 256: return run_csr<Pol, 8>(A, p, alpha, x, beta, y, flags, w, st);
+      case 512: return run_csr<Pol, 16>(A, p, alpha, x, beta, y, flags, w, st);
+      default: return run_csr<Pol, 32>(A, p, alpha, x, beta, y, flags, w, st);
+    }
+  };
+  switch (A->val_dtype) {
+    case MSREP_F64: return run(PolF64{});
+    case MSREP_F32: return run(PolF32<float>{});
+    default: return run(PolF32<bf16_t>{});
+  }
+}
+
 __global__ void scale_any(void *y, int64_t m, double beta, int is_f64) {
   for (int64_t r = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; r < m;
        r += int64_t(gridDim.x) * blockDim.x) {
