@@ -254,7 +254,8 @@ msrep_status msrep_spmv_workspace_size(const msrep_matrix *A,
  * or BF16 with xy_dtype F32 (the low-precision form: FP32 products, FP32
  * accumulation with TwoSum compensation: of rows longer than 256 nonzeros and
  * of rows split between thread-block tiles always, and in this version of
- * every row; partial sums of split rows merged in FP64).  x has n entries, y has m entries, device memory.
+ * every row; partial sums of split rows merged in FP64).  x has n entries, y
+ * has m entries, device memory.
  *
  * Merge: every row split by a partition (or tile) boundary gets
  * alpha * (sum of its partials, in partition order) + beta * y_in, beta
@@ -295,8 +296,8 @@ msrep_status msrep_spmm_workspace_size(const msrep_matrix *A, const msrep_partit
  * workspace with their values of each row side by side, so that each
  * nonzero gathers one segment for all of them and A is read once per pass
  * (ceil(k / 8) times in all).  A pass of one vector is msrep_spmv's, on x in
- * place or, where y overlaps it, on its copy.  Every column of Y is computed exactly as
- * msrep_spmv computes y for that x (same order of operations,
+ * place or, where y overlaps it, on its copy.  Every column of Y is computed
+ * exactly as msrep_spmv computes y for that x (same order of operations,
  * bit-identical results).  `flags`: MSREP_COMP_ALL / MSREP_COMP_NONE as
  * for msrep_spmv.  Asynchronous on `stream`.
  * Errors: INVALID_ARG (format not CSR, k < 1, ldx < n, ldy < m,
