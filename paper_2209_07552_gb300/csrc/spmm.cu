@@ -55,9 +55,18 @@ __global__ void __launch_bounds__(kKvThreads, KvShape<typename Pol::X, KP>::kBlo
   __shared__ KvWarpSmem<X, KvShape<X, KP>::VW> sm[kKvWarps];
   grid_dependency_wait();
   const int T = *n_tiles, wid = threadIdx.x >> 5;
+  const int first = blockIdx.x * kKvWarps + wid, stride = gridDim.x * kKvWarps;
+  // Vectors that take two passes over a tile (FP64, 5 to 8 of them): side by
+  // side where the grid has a warp for each, instead of one after the other
+  // (300 rows of 6 nonzeros, 8 vectors, 12.9 -> 9.8 us).
+  constexpr int VW = KvShape<X, KP>::VW, kPasses = KP / VW;
+  const bool apart = kPasses > 1 && int64_t(T) * kPasses <= stride;
   with_modes<Pol>(a.finish, a.comp_mode, [&](auto copy, auto comp) {
-    for (int b = blockIdx.x * kKvWarps + wid; b < T; b += gridDim.x * kKvWarps)
-      kv_tile<Pol, KP, decltype(copy)::value, decltype(comp)::value>(a, b, a.nnz, sm[wid]);
+    for (int i = first; i < (apart ? T * kPasses : T); i += stride) {
+      const int vb = apart ? i / T * VW : 0;
+      kv_tile<Pol, KP, decltype(copy)::value, decltype(comp)::value>(
+          a, apart ? i % T : i, a.nnz, sm[wid], vb, apart ? vb + VW : KP);
+    }
   });
 }
 
@@ -159,8 +168,8 @@ static msrep_status run_spmm(const msrep_matrix *A, const msrep_partition *p, in
   const int32_t *n_tiles = reinterpret_cast<const int32_t *>(plan + L.off_toff) + p->np;
   int nb = 1;
   MSREP_TRY(blocks_of(csr_spmm_direct<Pol, KP>, 0, KvShape<X, KP>::kBlocks, &nb));
-  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.tmax, kKvWarps),
-                                                             int64_t(nb) * sm_count()));
+  const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(
+      ceil_div(L.tmax * (KP / KvShape<X, KP>::VW), kKvWarps), int64_t(nb) * sm_count()));
   MSREP_TRY(launch_dependent(csr_spmm_direct<Pol, KP>, grid, kKvThreads, st, 0, a, n_tiles));
   CsrTileView v{a.tile_row, a.tile_k, A->ptr, n_tiles};
   const int64_t fg =

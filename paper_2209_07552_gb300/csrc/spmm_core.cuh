@@ -341,11 +341,13 @@ __device__ __forceinline__ void load4(const T *arr, int32_t h4, int32_t nnz, U (
   }
 }
 
-// Tile b by one warp.  kCopy: alpha = 1, beta = 0 known at compile time;
-// kComp: compensated sums (low-precision form).
+// Vectors [vb, ve) (a multiple of VW) of tile b by one warp.  kCopy: alpha = 1,
+// beta = 0 known at compile time; kComp: compensated sums (low-precision
+// form).
 template <class Pol, int KP, bool kCopy, bool kComp>
-__device__ __forceinline__ void kv_tile(const SpmmArgs<Pol> &a, int b, int32_t nnz,
-                                        KvWarpSmem<typename Pol::X, KvShape<typename Pol::X, KP>::VW> &sm) {
+__device__ __forceinline__ void kv_tile(
+    const SpmmArgs<Pol> &a, int b, int32_t nnz,
+    KvWarpSmem<typename Pol::X, KvShape<typename Pol::X, KP>::VW> &sm, int vb = 0, int ve = KP) {
   using X = typename Pol::X;
   using LV = typename LoadT<typename Pol::V>::type;
   constexpr int VW = KvShape<X, KP>::VW;
@@ -411,13 +413,13 @@ __device__ __forceinline__ void kv_tile(const SpmmArgs<Pol> &a, int b, int32_t n
   }
 
   // rows [w0, w0 + kKvRows) of the row ends, vectors [v0, v0 + VW)
-  for (int w0 = 0, v0 = 0; v0 < KP;) {
+  for (int w0 = 0, v0 = vb; v0 < ve;) {
     // --- the lane's nonzeros
     const X *xb = a.xt + v0;
     Acc acc;
     acc.zero();
     int rank = rank0 - w0;
-    if ((v0 > 0 || w0 > 0) && h_lo < h_hi) {
+    if ((v0 > vb || w0 > 0) && h_lo < h_hi) {
       load4(a.col_idx, h_lo * 4, nnz, cn);
       load4(a.val, h_lo * 4, nnz, vn);
     }
