@@ -45,16 +45,19 @@ msrep_status launch_batched(const BatchItem *items, const int64_t *toff, int cou
 // with the x interleaved by width spmm_width(k_j)), ys[j] = its k_j y
 // vectors of m_j values.  Tiles numbered by toff as for launch_batched;
 // uoff (count+1 entries, device) numbers the block work units, item j
-// having batched_k_units(tiles_j, k_j) of them, total_units in all; head,
+// having batched_k_units(tiles_j) of them, total_units in all; head,
 // tail: total_tiles * kBatchWidth doubles each.  y = A x for every vector
 // (alpha 1, beta 0).  Asynchronous.
 msrep_status launch_batched_k(const BatchItem *items, const int64_t *toff, const int64_t *uoff,
                               int count, int64_t total_tiles, int64_t total_units,
                               const void *const *xin, void *const *xt, void *const *ys,
-                              double *head, double *tail, unsigned flags, cudaStream_t st);
+                              double *head, double *tail, bool short_rows, cudaStream_t st);
 
-// block work units of an item of `tiles` tiles and k vectors in the
-// batched k-vector kernel
-int64_t batched_k_units(int64_t tiles, int k);
+// block work units of an item of `tiles` tiles in the batched k-vector kernel
+int64_t batched_k_units(int64_t tiles);
+
+// Are the item's rows so short, for its tile, that the kernel's form for short
+// rows does better?  (short_rows above: most tiles are such items'.)
+bool batched_k_short(const BatchItem &it, int32_t tile);
 
 }  // namespace msrep

@@ -281,7 +281,7 @@ static msrep_status launch_context(msrep_server *s, Context &c,
   void **xtp = reinterpret_cast<void **>(dp + L.xtp);
   void **ysk = reinterpret_cast<void **>(dp + L.ysk);
 
-  int64_t xo = 0, yo = 0, xto = 0, tt = 0, ttk = 0, utk = 0;
+  int64_t xo = 0, yo = 0, xto = 0, tt = 0, ttk = 0, utk = 0, stk = 0;
   int n1 = 0, nk = 0, nci = 0, nco = 0;
   c.y_off.clear();
   MSREP_CUDA_TRY(cudaEventRecord(c.begin_ev, c.stream));
@@ -322,7 +322,8 @@ static msrep_status launch_context(msrep_server *s, Context &c,
       toffk[nk] = ttk;
       uoffk[nk] = utk;
       ttk += rtiles[i];
-      utk += batched_k_units(rtiles[i], r->k);
+      utk += batched_k_units(rtiles[i]);
+      if (batched_k_short(itk[nk], effective_tile(s->cfg.tile))) stk += rtiles[i];
       xin[nk] = xsrc;
       xtp[nk] = c.xt_dev + xto;
       ysk[nk] = ydst;
@@ -351,8 +352,8 @@ static msrep_status launch_context(msrep_server *s, Context &c,
                                reinterpret_cast<const int64_t *>(dd + L.uoffk), nk, ttk, utk,
                                reinterpret_cast<const void *const *>(dd + L.xin),
                                reinterpret_cast<void *const *>(dd + L.xtp),
-                               reinterpret_cast<void *const *>(dd + L.ysk), c.head_k, c.tail_k, 0,
-                               c.stream));
+                               reinterpret_cast<void *const *>(dd + L.ysk), c.head_k, c.tail_k,
+                               2 * stk > ttk, c.stream));
   MSREP_CUDA_TRY(cudaEventRecord(c.k1_ev, c.stream));
   MSREP_TRY(launch_copies(reinterpret_cast<const CopyItem *>(dd + L.cin) + (R - nco), nco,
                           c.stream));

@@ -48,23 +48,23 @@ __global__ void interleave_x(const X *x, int64_t ldx, int k, int64_t n, X *xt) {
     interleave_column<X, KP>(x, ldx, k, c, xt);
 }
 
-template <class Pol, int KP>
+template <class Pol, int KP, bool kShort>
 __global__ void __launch_bounds__(kKvThreads, KvShape<typename Pol::X, KP>::kBlocks)
     csr_spmm_direct(SpmmArgs<Pol> a, const int32_t *n_tiles) {
   using X = typename Pol::X;
-  __shared__ KvWarpSmem<X, KvShape<X, KP>::VW> sm[kKvWarps];
+  __shared__ KvWarpSmem<X, KvShape<X, KP>::VW, kShort> sm[kKvWarps];
   grid_dependency_wait();
   const int T = *n_tiles, wid = threadIdx.x >> 5;
   const int first = blockIdx.x * kKvWarps + wid, stride = gridDim.x * kKvWarps;
   // Vectors that take two passes over a tile (FP64, 5 to 8 of them): side by
   // side where the grid has a warp for each, instead of one after the other
-  // (300 rows of 6 nonzeros, 8 vectors, 12.9 -> 9.8 us).
+  // (300 rows of 6 nonzeros, 8 vectors, 12.7 -> 9.8 us).
   constexpr int VW = KvShape<X, KP>::VW, kPasses = KP / VW;
   const bool apart = kPasses > 1 && int64_t(T) * kPasses <= stride;
   with_modes<Pol>(a.finish, a.comp_mode, [&](auto copy, auto comp) {
     for (int i = first; i < (apart ? T * kPasses : T); i += stride) {
       const int vb = apart ? i / T * VW : 0;
-      kv_tile<Pol, KP, decltype(copy)::value, decltype(comp)::value>(
+      kv_tile<Pol, KP, decltype(copy)::value, decltype(comp)::value, kShort>(
           a, apart ? i % T : i, a.nnz, sm[wid], vb, apart ? vb + VW : KP);
     }
   });
@@ -167,10 +167,12 @@ static msrep_status run_spmm(const msrep_matrix *A, const msrep_partition *p, in
   a.comp_mode = flags & (MSREP_COMP_ALL | MSREP_COMP_NONE);
   const int32_t *n_tiles = reinterpret_cast<const int32_t *>(plan + L.off_toff) + p->np;
   int nb = 1;
-  MSREP_TRY(blocks_of(csr_spmm_direct<Pol, KP>, 0, KvShape<X, KP>::kBlocks, &nb));
+  const auto kern = kv_short_rows(A->m, A->nnz, tile) ? csr_spmm_direct<Pol, KP, true>
+                                                     : csr_spmm_direct<Pol, KP, false>;
+  MSREP_TRY(blocks_of(kern, 0, KvShape<X, KP>::kBlocks, &nb));
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(
       ceil_div(L.tmax * (KP / KvShape<X, KP>::VW), kKvWarps), int64_t(nb) * sm_count()));
-  MSREP_TRY(launch_dependent(csr_spmm_direct<Pol, KP>, grid, kKvThreads, st, 0, a, n_tiles));
+  MSREP_TRY(launch_dependent(kern, grid, kKvThreads, st, 0, a, n_tiles));
   CsrTileView v{a.tile_row, a.tile_k, A->ptr, n_tiles};
   const int64_t fg =
       std::max<int64_t>(1, std::min<int64_t>(ceil_div(L.tmax * KP, 256), 8 * sm_count()));
@@ -235,14 +237,15 @@ __device__ __forceinline__ int owner_item_k(const int64_t *toff, int count, int6
 // units of kKvWarps tiles, one unit per block at a time, one tile per warp.
 // The warps never wait for one another.
 // The item's pointers are kept in shared memory: in registers they spilled.
-template <class Pol, bool kComp>
+template <class Pol, bool kShort>
 __global__ void __launch_bounds__(kKvThreads, 4)
     batched_spmm(const BatchItem *items, const int64_t *toff, const int64_t *uoff, int count,
                  const void *const *xs, void *const *ys, double *head, double *tail) {
   using X = typename Pol::X;
-  using Slot = KvWarpSmem<X, KvShape<X, 8>::VW>;  // the widest layout's
-  static_assert(sizeof(KvWarpSmem<X, KvShape<X, 2>::VW>) <= sizeof(Slot) &&
-                    sizeof(KvWarpSmem<X, KvShape<X, 4>::VW>) <= sizeof(Slot),
+  using Smem2 = KvWarpSmem<X, KvShape<X, 2>::VW, kShort>;
+  using Smem4 = KvWarpSmem<X, KvShape<X, 4>::VW, kShort>;
+  using Slot = KvWarpSmem<X, KvShape<X, 8>::VW, kShort>;
+  static_assert(sizeof(Smem2) <= sizeof(Slot) && sizeof(Smem4) <= sizeof(Slot),
                 "every layout fits the widest one's slot");
   __shared__ Slot sm[kKvWarps];
   __shared__ SpmmArgs<Pol> s_args[kKvWarps];
@@ -289,13 +292,11 @@ __global__ void __launch_bounds__(kKvThreads, 4)
     }
     const int kp = spmm_width(a.k);
     if (kp == 2)
-      kv_tile<Pol, 2, true, kComp>(
-          a, b, a.nnz, *reinterpret_cast<KvWarpSmem<X, KvShape<X, 2>::VW> *>(sm + wid));
+      kv_tile<Pol, 2, true, Pol::kLow, kShort>(a, b, a.nnz, *reinterpret_cast<Smem2 *>(sm + wid));
     else if (kp == 4)
-      kv_tile<Pol, 4, true, kComp>(
-          a, b, a.nnz, *reinterpret_cast<KvWarpSmem<X, KvShape<X, 4>::VW> *>(sm + wid));
+      kv_tile<Pol, 4, true, Pol::kLow, kShort>(a, b, a.nnz, *reinterpret_cast<Smem4 *>(sm + wid));
     else
-      kv_tile<Pol, 8, true, kComp>(a, b, a.nnz, sm[wid]);
+      kv_tile<Pol, 8, true, Pol::kLow, kShort>(a, b, a.nnz, sm[wid]);
   }
 }
 
@@ -350,20 +351,23 @@ __global__ void interleave_batch(const BatchItem *items, int count, const void *
   }
 }
 
-int64_t batched_k_units(int64_t tiles, int) { return (tiles + kKvWarps - 1) / kKvWarps; }
+int64_t batched_k_units(int64_t tiles) { return (tiles + kKvWarps - 1) / kKvWarps; }
+
+bool batched_k_short(const BatchItem &it, int32_t tile) {
+  return kv_short_rows(it.m, it.nnz, tile);
+}
 
 msrep_status launch_batched_k(const BatchItem *items, const int64_t *toff, const int64_t *uoff,
                               int count, int64_t total_tiles, int64_t total_units,
                               const void *const *xin, void *const *xt, void *const *ys,
-                              double *head, double *tail, unsigned flags, cudaStream_t st) {
+                              double *head, double *tail, bool short_rows, cudaStream_t st) {
   if (count == 0) return MSREP_OK;
   const int sms = sm_count();
   interleave_batch<float><<<dim3(64, std::min(count, 1024)), 256, 0, st>>>(items, count, xin, xt);
   MSREP_CUDA_TRY(cudaGetLastError());
   if (total_tiles == 0) return MSREP_OK;
-  const auto kern = (flags & (MSREP_COMP_ALL | MSREP_COMP_NONE)) == MSREP_COMP_NONE
-                        ? batched_spmm<PolF32<float>, false>
-                        : batched_spmm<PolF32<float>, true>;
+  const auto kern = short_rows ? batched_spmm<PolF32<float>, true>
+                               : batched_spmm<PolF32<float>, false>;
   int nb = 1;
   MSREP_TRY(blocks_of(kern, 0, 4, &nb));
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(total_units, int64_t(nb) * sms));

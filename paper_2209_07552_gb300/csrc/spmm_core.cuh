@@ -74,22 +74,46 @@ constexpr int kKvThreads = 32 * kKvWarps;
 constexpr int kKvBitWords = 34;   // a tile of <= 1024 nonzeros in aligned groups of 8
 constexpr int kKvRows = 88;       // rows of the row buffer
 
+// Is kShort the better form of kv_tile (see there)?  Where the mean tile has
+// clearly more row ends than the row buffer holds.  Rows without nonzeros end
+// at none, and how many there are the call does not know: with fewer nonzeros
+// than rows most are taken to be such.
+inline bool kv_short_rows(int64_t m, int64_t nnz, int32_t tile) {
+  return nnz >= m && m * tile > (m + nnz) * (kKvRows + 12);
+}
+
 // Shared memory of one warp.  A stored accumulator is VW sums, then (FP32)
 // their VW compensations; 16 bytes of padding from 32 bytes on let a warp
 // read one per lane without bank conflicts.
-template <class X, int VW>
+template <class X, int VW, bool kShort = false>
 struct KvWarpSmem {
   static constexpr int kAcc = (sizeof(X) == 4 ? 2 : 1) * VW;
   static constexpr int kSlot = kAcc * int(sizeof(X)) >= 32 ? kAcc + 16 / int(sizeof(X)) : kAcc;
-  // finished rows' accumulators in the order of the rows' ends.  kKvRows
-  // holds every tile of 512 whose rows average five nonzeros; a tile with
-  // more row ends is walked once for each kKvRows of them.
-  alignas(16) X rows[kKvRows][kSlot];
+  // finished rows' accumulators in the order of the rows' ends
+  static constexpr int kRows = !kShort                   ? kKvRows
+                               : kSlot * sizeof(X) == 16 ? 256
+                               : sizeof(X) == 8          ? 192
+                                                         : 144;
+  alignas(16) X rows[kRows][kSlot];
   alignas(16) X last[kAcc];          // the row that continues past the tile
   uint32_t end[kKvBitWords];         // bit e: a row ends with element e of the tile
+  // A tile written directly (kv_tile): the rows that hold a nonzero and end in
+  // it, at most 512 of a tile of 1024 items, behind a slot or two a lane.
+  static constexpr bool kSpare = sizeof(X) == 4 && VW > 2;
+  static constexpr int kList = kSpare ? 64 : 32;
+  static_assert(!kShort || (kRows - kList) * kSlot * sizeof(X) >= 512 * sizeof(uint16_t),
+                "room for the list");
+  __device__ __forceinline__ uint16_t *row_of() { return reinterpret_cast<uint16_t *>(rows[kList]); }
 };
 
-// Vector j of a stored accumulator as the FP64 partial of a split row.
+// Vector j of a stored accumulator: the total that y takes, and the FP64
+// partial of a split row.
+template <int VW>
+__device__ __forceinline__ double kv_total(const double *p, int j) { return p[j]; }
+template <int VW>
+__device__ __forceinline__ float kv_total(const float *p, int j) {
+  return pair_total(p[j], p[VW + j]);
+}
 template <int VW>
 __device__ __forceinline__ double kv_partial(const double *p, int j) { return p[j]; }
 template <int VW>
@@ -344,10 +368,22 @@ __device__ __forceinline__ void load4(const T *arr, int32_t h4, int32_t nnz, U (
 // Vectors [vb, ve) (a multiple of VW) of tile b by one warp.  kCopy: alpha = 1,
 // beta = 0 known at compile time; kComp: compensated sums (low-precision
 // form).
-template <class Pol, int KP, bool kCopy, bool kComp>
+//
+// A tile with more row ends than the row buffer holds is walked once for each
+// kKvRows of them.  kShort: the buffer is larger (the loop then has less L1 for
+// x), and a tile beyond it is walked once too, its rows written from the nonzero
+// loop, all but each lane's first, which waits for its carry in the lane's slot
+// (the wider FP32 layouts through another slot of the lane: from registers the
+// stores spilled).  The loop pays a few percent for that choice at each row
+// end, so kShort is taken where the mean tile needs it (kv_short_rows).
+// Measured without -> with, tile 512: rows of three nonzeros FP64 k = 4 67 -> 47
+// us, FP32 k = 2 34 -> 24; of two 80 -> 59 and 37 -> 27; of one 146 -> 116 and 58
+// -> 40; Laplacian 2048^2 with tile 1024, FP64 k = 4, 437 -> 283.
+template <class Pol, int KP, bool kCopy, bool kComp, bool kShort = false>
 __device__ __forceinline__ void kv_tile(
     const SpmmArgs<Pol> &a, int b, int32_t nnz,
-    KvWarpSmem<typename Pol::X, KvShape<typename Pol::X, KP>::VW> &sm, int vb = 0, int ve = KP) {
+    KvWarpSmem<typename Pol::X, KvShape<typename Pol::X, KP>::VW, kShort> &sm, int vb = 0,
+    int ve = KP) {
   using X = typename Pol::X;
   using LV = typename LoadT<typename Pol::V>::type;
   constexpr int VW = KvShape<X, KP>::VW;
@@ -412,13 +448,52 @@ __device__ __forceinline__ void kv_tile(
     rank0 = inc - cnt;
   }
 
-  // rows [w0, w0 + kKvRows) of the row ends, vectors [v0, v0 + VW)
+  using Smem = KvWarpSmem<X, VW, kShort>;
+  constexpr int kRows = Smem::kRows;
+  const bool direct = kShort && ends > kRows;
+  uint16_t *row_of = sm.row_of();
+  if (direct) {
+    int before = 0;
+    for (int i0 = 0; i0 < nrows; i0 += 32) {
+      const int i = i0 + lane;
+      const int32_t st = i < nrows ? __ldg(a.row_ptr + r0 + i) : 0;
+      const int32_t en = i < nrows ? __ldg(a.row_ptr + r0 + i + 1) : 0;
+      const bool holds = i < nrows && en > max(st, k0);
+      const unsigned dm = __ballot_sync(full, holds);
+      if (holds) row_of[before + __popc(dm & ((1u << lane) - 1u))] = static_cast<uint16_t>(i);
+      before += __popc(dm);
+    }
+    __syncwarp();
+  }
+  auto write_row = [&](int v0, int32_t i, const Acc &tot, X *p) {
+    X *yp = a.y + v0 * a.ldy + r0 + i;
+    if constexpr (Smem::kSpare) {
+      tot.store(p);
+#pragma unroll 1
+      for (int j = 0; j < VW && v0 + j < a.k; ++j, yp += a.ldy)
+        *yp = finish_total(kv_total<VW>(p, j), fin, a.alpha, a.beta, yp);
+    } else {
+      X t[VW];
+      tot.totals(t);
+#pragma unroll
+      for (int j = 0; j < VW; ++j)
+        if (v0 + j < a.k)
+          yp[j * a.ldy] = finish_total(t[j], fin, a.alpha, a.beta, yp + j * a.ldy);
+    }
+  };
+
+  // rows [w0, w0 + kRows) of the row ends (all of them if direct), vectors
+  // [v0, v0 + VW)
   for (int w0 = 0, v0 = vb; v0 < ve;) {
     // --- the lane's nonzeros
     const X *xb = a.xt + v0;
     Acc acc;
     acc.zero();
-    int rank = rank0 - w0;
+    // slot of the lane's next row end: its rank in the window, or, written
+    // directly, `lane` and then none (its ends counted in steps of kPast)
+    constexpr int kPast = 1 << 20;
+    const int slot0 = direct ? lane : rank0 - w0, step = direct ? kPast : 1;
+    int slot = slot0;
     if ((v0 > vb || w0 > 0) && h_lo < h_hi) {
       load4(a.col_idx, h_lo * 4, nnz, cn);
       load4(a.val, h_lo * 4, nnz, vn);
@@ -445,15 +520,22 @@ __device__ __forceinline__ void kv_tile(
       for (int u = 0; u < 4; ++u) {
         if ((in >> u) & 1u) acc.template fma<kComp>(v[u], x[u]);
         if ((eb >> u) & 1u) {  // a row ends here
-          if (static_cast<unsigned>(rank) < unsigned(kKvRows)) acc.store(sm.rows[rank]);
-          ++rank;
+          if constexpr (kShort) {
+            if (slot < kRows)
+              acc.store(sm.rows[slot]);
+            else
+              write_row(v0, row_of[rank0 + slot / kPast], acc, sm.rows[32 + lane]);
+          } else {
+            if (static_cast<unsigned>(slot) < unsigned(kRows)) acc.store(sm.rows[slot]);
+          }
+          slot += step;
           acc.zero();
         }
       }
     }
 
     // --- rows split between lanes: warp_seg_scan's doubling, for all VW
-    const bool emitted = rank > rank0 - w0;
+    const bool emitted = slot != slot0;
     bool f = emitted;
 #pragma unroll 1
     for (int o = 1; o < 32; o <<= 1) {
@@ -467,12 +549,16 @@ __device__ __forceinline__ void kv_tile(
     }
     Acc ex = acc.shfl_up(1);
     if (lane == 0) ex.zero();
-    if (emitted && static_cast<unsigned>(rank0 - w0) < unsigned(kKvRows)) {
+    if (emitted && static_cast<unsigned>(slot0) < unsigned(kRows)) {
       Acc tot;
-      tot.load(sm.rows[rank0 - w0]);
+      tot.load(sm.rows[slot0]);
       tot.carry_in(ex);
-      tot.store(sm.rows[rank0 - w0]);
+      if (direct && !(rank0 == 0 && has0 && flag))
+        write_row(v0, row_of[rank0], tot, sm.rows[lane]);
+      else
+        tot.store(sm.rows[slot0]);
     }
+    const unsigned em = kShort && direct ? __ballot_sync(full, emitted) : 1u;
     if (lane == 31) acc.store(sm.last);
     __syncwarp();
 
@@ -482,7 +568,7 @@ __device__ __forceinline__ void kv_tile(
     // the last row's.  A first row that ended where the tile starts adds 0.
     if (w0 == 0) {
       const int j = lane & 15;
-      const X *src = lane < 16 ? sm.rows[0] : sm.last;
+      const X *src = lane < 16 ? sm.rows[__ffs(em) - 1] : sm.last;
       double *dst = nullptr;
       if (lane < 16) {
         if (flag && nrows > 0) dst = a.head;
@@ -510,7 +596,7 @@ __device__ __forceinline__ void kv_tile(
       const int rk = done + __popc(dm & ((1u << lane) - 1u));
       done += __popc(dm);
       if (valid && !(i == 0 && flag) &&
-          (holds ? static_cast<unsigned>(rk) < unsigned(kKvRows) : w0 == 0)) {
+          (holds ? !direct && static_cast<unsigned>(rk) < unsigned(kRows) : w0 == 0)) {
         X t[VW];
         if (holds) {
           Acc tot;
@@ -528,8 +614,8 @@ __device__ __forceinline__ void kv_tile(
       }
     }
     __syncwarp();
-    w0 += kKvRows;
-    if (w0 >= ends) {
+    w0 += kRows;
+    if (direct || w0 >= ends) {
       w0 = 0;
       v0 += VW;
     }
