@@ -236,7 +236,8 @@ __device__ __forceinline__ int owner_item_k(const int64_t *toff, int count, int6
 // spmm_width(k_j) and its tiles cut into uoff[j+1] - uoff[j] block work
 // units of kKvWarps tiles, one unit per block at a time, one tile per warp.
 // The warps never wait for one another.
-// The item's pointers are kept in shared memory: in registers they spilled.
+// The item's pointers are kept in shared memory: in registers more would spill
+// (the kernel stores 146 bytes and loads 184 as it is).
 template <class Pol, bool kShort>
 __global__ void __launch_bounds__(kKvThreads, 4)
     batched_spmm(const BatchItem *items, const int64_t *toff, const int64_t *uoff, int count,

@@ -1,25 +1,25 @@
 // k right-hand sides at once (Y = alpha * A * X + beta * Y, k <= 8) over
 // the same CSR tiles as the SpMV: the served form's sweep of up to eight x
 // vectors per request.  X is read interleaved, row c of X holding the KP
-// values x_0[c] .. x_{KP-1}[c] (KP = k rounded up to 1, 2, 4 or 8), so a
-// nonzero gathers one contiguous 4..64-byte segment, and the matrix is
+// values x_0[c] .. x_{KP-1}[c] (KP = k rounded up to 2, 4 or 8), so a
+// nonzero gathers one contiguous 8..64-byte segment, and the matrix is
 // streamed once for all k vectors.
 //
 // One warp works on a tile alone, lane l walking exactly the nonzeros that
 // lane l of the SpMV's warp walks, with the same FMAs in the same order for
-// each vector (masked positions add zero) and the same warp scan, so
-// Y[:, v] equals msrep_spmv of x_v bit for bit.  A lane holds VW vectors: up
-// to 32 bytes of an x row, fetched by one 256-bit load (FP64 with eight
-// vectors takes two passes over the tile).
+// each vector and the same warp scan, so Y[:, v] equals msrep_spmv of x_v bit
+// for bit.  A lane holds VW vectors: up to 32 bytes of an x row, fetched by one
+// 256-bit load (FP64 with eight vectors takes two passes over the tile).  One
+// vector takes the SpMV kernels themselves.
 //
 // What bounds it: one L1 line lookup per nonzero for the gather (16.8M of
 // them take about 55 us on 152 SMs) and, above that, the instructions around
 // it at 16 warps an SM (87M warp instructions on the R-MAT matrix, k = 8;
-// issue slots 46% used, L1 60%).  Measured on R-MAT 2^20 / 2^24 nonzeros,
-// FP32, the whole call: k = 2 / 4 / 8 108 / 135 / 206 us, against 186 / 345 /
+// issue slots 46% used, L1 65%).  Measured on R-MAT 2^20 / 2^24 nonzeros,
+// FP32, the whole call: k = 2 / 4 / 8 110 / 132 / 208 us, against 186 / 345 /
 // 539 us with row ends walked inside the nonzero loop and y written from
-// there (197M warp instructions at k = 8); 2048^2 Laplacian k = 8 290 against
-// 481 us.  Three things keep the instructions few:
+// there (197M warp instructions at k = 8); 2048^2 Laplacian k = 8 293 against
+// 508 us.  Three things keep the instructions few:
 //  * where the rows of the tile end is worked out once per tile, a lane per
 //    row, into a bit string in shared memory; the nonzero loop tests one bit
 //    instead of walking row pointers on a divergent path;
@@ -53,7 +53,7 @@ struct SpmmArgs {
   unsigned comp_mode;
 };
 
-// KP of a request of k vectors: k rounded up to 1, 2, 4 or 8
+// width of the interleaved x of k vectors: k rounded up to 1, 2, 4 or 8
 __host__ __device__ constexpr int spmm_width(int k) {
   return k <= 1 ? 1 : k <= 2 ? 2 : k <= 4 ? 4 : 8;
 }
@@ -63,9 +63,8 @@ template <class X, int KP>
 struct KvShape {
   static constexpr int VW = KP * int(sizeof(X)) <= 32 ? KP : 32 / int(sizeof(X));
   // Resident blocks (of 4 warps) per SM asked of the register allocator: 32
-  // bytes of x a lane need about 120 registers, and five blocks (96, with
-  // spills) took 215 us where four take 207 (R-MAT, FP32, k = 8); the
-  // narrower ones fit more.
+  // bytes of x a lane need 128 registers, and five blocks (96, with spills) took
+  // 215 us where four take 207 (R-MAT, FP32, k = 8); the narrower ones fit more.
   static constexpr int kBlocks = VW * int(sizeof(X)) == 32 ? 4 : VW * int(sizeof(X)) == 16 ? 6 : 7;
 };
 

@@ -248,9 +248,9 @@ __global__ void __launch_bounds__(kThreads) csr_stream(CsrArgs<Pol> a, const int
     fill_tail(val_s(s), a.val, v, v.base, g_end);
     __syncwarp();
     with_modes<Pol>(kFinishScale, a.comp_mode, [&](auto, auto comp) {
-      csr_tile_compute<Pol, SharedSrc, false, decltype(comp)::value>(
+      csr_tile_compute<Pol, decltype(comp)::value>(
           a, b, c.x, c.y, c.z, c.w, rp_s(s) + (c.x - p.base), Seg<int32_t>{col_s(s), q.base},
-          Seg<V>{val_s(s), v.base}, nnz, SharedSrc{});
+          Seg<V>{val_s(s), v.base}, nnz);
     });
     __syncwarp();
     if (lane == 0 && b + S * W < T) {

@@ -354,22 +354,19 @@ struct RowChunks {
 // pointers it has staged; the same sums.
 // One merge-path tile b = rows [r0, r1] x nonzeros [k0, k1), processed by
 // one warp.  rp[j] = row_ptr[r0 + j] for j = 0..r1-r0, and also j = r1-r0+1
-// when r1 < m; rp must be in shared memory (it is searched).
-// kCopy: the caller knows that alpha = 1 and beta = 0 (every row finished
-// by the copy mode, decided at compile time).  kComp: compensated sums
+// when r1 < m; rp, col and val are in shared memory.  kComp: compensated sums
 // (low-precision form).
-template <class Pol, class Src, bool kCopy, bool kComp>
+template <class Pol, bool kComp>
 __device__ __forceinline__ void csr_tile_compute(const CsrArgs<Pol> &a, int b, int32_t r0,
                                                  int32_t k0, int32_t r1, int32_t k1,
                                                  const int32_t *rp, Seg<int32_t> col,
-                                                 Seg<typename Pol::V> val, int64_t nnz,
-                                                 Src src) {
+                                                 Seg<typename Pol::V> val, int64_t nnz) {
   using Acc = typename Pol::Acc;
   using LV = typename LoadT<typename Pol::V>::type;
   const int lane = threadIdx.x & 31;
-  const int fin = kCopy ? int(kFinishCopy) : a.finish;
+  const SharedSrc src{};
   auto write_row_k = [&](int32_t row, Acc v) {
-    a.y[row] = Pol::finish(v, fin, a.alpha, a.beta, a.y + row);
+    a.y[row] = Pol::finish(v, a.finish, a.alpha, a.beta, a.y + row);
   };
   const int nrows = r1 - r0;
   const int32_t rs0 = rp[0];
