@@ -335,7 +335,7 @@ struct TileLen {
 // partitions, 32 at a time; its loads are all in flight at once.  The sums fit
 // 32 bits: at most 2^31 + 2 np local entries, and fewer tiles.
 constexpr int kFillThreads = 256;
-constexpr int kScanMax = 4096;
+constexpr int kScanMax = 3072;
 template <class Len>
 __device__ __forceinline__ void block_offsets(int32_t np, Len len, uint32_t *s_off) {
   constexpr int kWarps = kFillThreads / 32, kRows = kScanMax / kFillThreads;
@@ -542,31 +542,50 @@ __global__ void __launch_bounds__(256)
 // A thread per tile t: its partition is the last i with off(i) <= t (a
 // partition without tiles shares its offset with the next), its diagonal the
 // g-th even cut of that partition's stretch.  (A block per partition left a
-// matrix in one partition to 128 threads: 462 us for 2^24 nonzeros.)
+// matrix in one partition to 128 threads: 462 us for 2^24 nonzeros.)  The warp
+// searches for its first tile's partition; its tiles lie in that one and the
+// next 31, unless some of those have no tiles, so their offsets are one more
+// load and a search among the lanes.  (A search by each thread was a dependent
+// load per bit of np: R-MAT 2^20 / 2^24, 2368 and 9472 partitions, plan alone,
+// 14.6 and 25.6 us, now 13.5 and 22.8 with the same launches.)
 template <class Off>
 __device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32_t n_major,
                                           int64_t nnz, int32_t np, const int64_t *D,
                                           const int32_t *R, Off off, int32_t *tile_row,
                                           int32_t *tile_k, int64_t t) {
-  const int64_t T = off(np);
-  if (t > T) return;
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t T = off(np), w0 = t - lane;
+  if (w0 > T) return;
   if (t == T) {
     tile_row[T] = n_major;
     tile_k[T] = static_cast<int32_t>(nnz);
-    return;
   }
-  int32_t lo = 0, hi = np - 1;
-  while (lo < hi) {
-    const int32_t mid = lo + (hi - lo + 1) / 2;
-    if (off(mid) <= t)
-      lo = mid;
-    else
-      hi = mid - 1;
+  if (w0 == T) return;  // warp-uniform, as the one above
+  const int32_t ia = last_le_warp_at(off, 0, np - 1, w0);
+  const int64_t mine = off(min(ia + 1 + lane, np));  // end of partition ia + lane
+  int j = 0;  // partitions from ia on that end at or before t, at most 31
+#pragma unroll
+  for (int step = 16; step; step /= 2)
+    if (__shfl_sync(full, mine, j + step - 1) <= t) j += step;
+  int32_t i = ia + j;
+  int64_t t1 = __shfl_sync(full, mine, j), t0 = __shfl_sync(full, mine, max(j - 1, 0));
+  if (t >= T) return;
+  if (j == 0) t0 = off(ia);
+  if (t1 <= t) {  // past the 32
+    int32_t hi = np - 1;
+    while (i < hi) {
+      const int32_t mid = i + (hi - i + 1) / 2;
+      if (off(mid) <= t)
+        i = mid;
+      else
+        hi = mid - 1;
+    }
+    t0 = off(i), t1 = off(i + 1);
   }
-  const int64_t t0 = off(lo), G = off(lo + 1) - t0;
-  const int64_t d0 = __ldg(D + lo), len = __ldg(D + lo + 1) - d0;
-  const int64_t d = d0 + ((t - t0) * len) / G;
-  const int32_t r = path_row(ptr, __ldg(R + lo), __ldg(R + lo + 1), d);
+  const int64_t d0 = __ldg(D + i), len = __ldg(D + i + 1) - d0;
+  const int64_t d = d0 + ((t - t0) * len) / (t1 - t0);
+  const int32_t r = path_row(ptr, __ldg(R + i), __ldg(R + i + 1), d);
   tile_row[t] = r;
   tile_k[t] = static_cast<int32_t>(d - r);
 }
@@ -577,10 +596,8 @@ __device__ __forceinline__ void plan_tile(const int32_t *__restrict__ ptr, int32
 // number, and the dependent loads in each, times a microsecond or so.
 // kScan: every block sums the lengths of all partitions itself, which takes
 // less than a launch between, and searches them in shared memory instead of a
-// dependent load per bit of np; the first block of each kind writes the offsets
-// out.  Otherwise part_scans has written them.  R-MAT 2^20 / 2^24 nonzeros, the
-// plan alone, 592 and 2368 partitions: 10.3 and 12.5 us, 12.9 and 14.6 with
-// part_scans; 2368 with local pointers 13.5 and 16.4.
+// chain of loads; the first block of each kind writes the offsets out.
+// Otherwise part_scans has written them.
 template <bool kVec, bool kScan>
 __global__ void __launch_bounds__(kFillThreads)
     part_fill(const int32_t *__restrict__ ptr, int32_t n_major, int64_t nnz, int32_t np,
@@ -588,7 +605,7 @@ __global__ void __launch_bounds__(kFillThreads)
               int32_t *tile_row, int32_t *tile_k, int plan_blocks, const int32_t *start_idx,
               const int32_t *end_idx, const int32_t *start_major, const int32_t *end_major,
               int64_t *local_off, int32_t *local) {
-  __shared__ uint32_t s_off[kScan ? kScanMax + 1 : 1];
+  extern __shared__ uint32_t s_off[];  // kScan: np + 1 offsets
   grid_dependency_wait();
   const int b = static_cast<int>(blockIdx.x);
   auto shared_off = [&](int32_t i) { return int64_t(s_off[i]); };
@@ -1034,11 +1051,14 @@ static msrep_status partition_compressed(const msrep_matrix *A,
       p->local ? static_cast<int>(std::max<int64_t>(
                      1, std::min<int64_t>(ceil_div(most, 8 * 256), 8 * sm_count())))
                : p->local_off ? 1 : 0;
-  // Every block scans (part_fill) where that takes less than a launch: up to
-  // 4096 partitions (R-MAT plan alone, 8192: 24.7 us against 22.8), and four
-  // blocks of local pointers an SM (R-MAT, 515 of them: 13.5 us against 16.4;
-  // Laplacian 2048^2, 1216: 23.6 against 21.8)
-  const bool scan = p->np <= kScanMax && fill_blocks <= 4 * sm_count();
+  // Every block scans (part_fill) where that takes less than a launch.  By
+  // partitions (R-MAT plan alone, part_scans / every block): 2368 13.5 / 12.7 us,
+  // 4096 15.4 / 15.8.  By plan blocks (rows of 100 nonzeros, 592 partitions):
+  // 155 9.7 / 8.2 us, 388 10.1 / 9.3, 542 10.9 / 10.7, 773 11.3 / 14.0.  By blocks
+  // of local pointers (2368 partitions): R-MAT, 515, 15.0 / 13.8 us; Laplacian
+  // 2048^2, 1216, 21.5 / 23.6.
+  const bool scan = p->np <= kScanMax && plan_blocks <= 3 * sm_count() &&
+                    fill_blocks <= 4 * sm_count();
   if (!scan && (toff || p->local_off))
     MSREP_TRY(launch_dependent(part_scans, toff && p->local_off ? 2 : 1, 1024, st, 0,
                                static_cast<const int32_t *>(p->start_major),
@@ -1050,7 +1070,8 @@ static msrep_status partition_compressed(const msrep_matrix *A,
                            : (vec ? part_fill<true, false> : part_fill<false, false>);
     int32_t *trow = plan ? reinterpret_cast<int32_t *>(plan + L.off_row) : nullptr;
     int32_t *tk = plan ? reinterpret_cast<int32_t *>(plan + L.off_k) : nullptr;
-    MSREP_TRY(launch_dependent(fill, plan_blocks + fill_blocks, kFillThreads, st, 0, A->ptr,
+    MSREP_TRY(launch_dependent(fill, plan_blocks + fill_blocks, kFillThreads, st,
+                               scan ? sizeof(uint32_t) * (size_t(p->np) + 1) : 0, A->ptr,
                                n_major, A->nnz, p->np, static_cast<const int64_t *>(D),
                                static_cast<const int32_t *>(R), tile, toff, trow, tk, plan_blocks,
                                p->start_idx, p->end_idx, p->start_major, p->end_major,

@@ -1,10 +1,11 @@
 """The tile plan of CSR and CSC partitions, entry for entry.
 
-Up to 4096 partitions every block of the plan sums the tiles of all partitions
-itself, 256 of them a row; beyond that, or with local pointers of over a million
-rows, a kernel before it does.  The cases lie on both sides of those limits,
-with partitions without tiles and with nearly all of them; the offsets of local
-pointers can be had alone.
+Up to 3072 partitions, and not too many tiles or rows, every block sums the
+lengths of all partitions itself, 256 of them a row; otherwise a kernel before
+it does.  A warp finds its first tile's partition and looks at the next 32.  The
+cases lie on both sides of those limits, with partitions without tiles and with
+nearly all of them; the offsets of local pointers can be had alone.
+
 All entries are integers and must equal the rule's: partition i spans the
 diagonals [D_i, D_i+1) of the merge path, cut into ceil(length / tile) even
 stretches, whose coordinates consume a row's end before the next nonzero.
@@ -67,7 +68,8 @@ def _got(part, P, m, nnz, tile):
 
 
 @pytest.mark.parametrize("name,m,nnz", [("ragged", 30000, 35500), ("ragged", 3000, 200000),
-                                        ("ends", 2600000, 3000), ("ends", 5000, 600),
+                                        ("ends", 2600000, 3000), ("ends", 40000000, 500),
+                                        ("ends", 5000, 600),
                                         ("ragged", 50, 7)])
 @pytest.mark.parametrize("fmt", ["csr", "csc"])
 def test_tile_plan(fmt, name, m, nnz):
@@ -75,7 +77,7 @@ def test_tile_plan(fmt, name, m, nnz):
     a = (_ragged if name == "ragged" else _sparse_ends)(m, nnz, seed=m)
     ptr = a.row_ptr if fmt == "csr" else I.csr_to_csc(a).col_ptr
     A = M.DeviceMatrix.from_host(a, fmt, "f64")
-    for P in (1, 2, 255, 256, 257, 1000, 4096, 4097, 6000):
+    for P in (1, 2, 31, 32, 33, 255, 256, 257, 1000, 3072, 3073, 6000) if m < 10**7 else (1, 592):
         for local in (False, True):
             part = M.DevicePartition(A, P, tile=256, local=local)
             part.plan.fill_(0x7f)      # what a caller's buffer may hold
