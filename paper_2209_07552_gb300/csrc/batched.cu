@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(BShape<W>::kThreads, BShape<W>::kMinBlocks)
       __syncwarp();
       if (lane == 0) {
         const BatchItem it = items[j];
+        a.part_toff = nullptr;
         a.row_ptr = it.row_ptr;
         a.col_idx = it.col_idx;
         a.val = static_cast<const typename Pol::V *>(it.val);
@@ -95,6 +96,8 @@ __global__ void __launch_bounds__(BShape<W>::kThreads, BShape<W>::kMinBlocks)
         a.head = head + base;
         a.tail = tail + base;
         a.m = it.m;
+        a.comp_mode = 0;
+        a.err = nullptr;
       }
       __syncwarp();
     }
